@@ -467,6 +467,7 @@ static cicero_status plan_batch(const cicero_job* jobs, int n_jobs, const cicero
       D.cam = view_of(J.cam);
       D.mlp = mlp_ptrs(J.mlp);
       D.density = J.grid->density;
+      D.features = J.grid->features;
       D.rgb = J.rgb;
       D.depth = J.depth;
       D.ray_base = (int)R;

@@ -170,6 +170,7 @@ struct JobDesc {  // aligned as CUtensorMap (64 bytes or more)
   ViewCam cam;
   MlpPtrs mlp;
   const void* density;
+  const void* features;
   float* rgb;        // [H*W][3]
   float* depth;      // [H*W] or NULL
   int ray_base;      // first ray of the job in the batch's ray numbering

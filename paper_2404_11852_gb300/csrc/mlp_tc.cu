@@ -23,6 +23,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -233,8 +234,7 @@ __device__ __forceinline__ bool mlp_tile(char* sm, Group& G, uint32_t* err, floa
 // View-direction encoding with the fast hardware sine/cosine (|d| <= 1, error ~1e-6, far below
 // the BF16 rounding of the MLP input) and the double-angle recurrence.
 template <int NF>
-__device__ __forceinline__ void encode_dir_fast(const float d[3], int n_freq_rt, float* x) {
-  const int n_freq = NF ? NF : n_freq_rt;
+__device__ __forceinline__ void encode_dir_fast(const float d[3], float* x) {
   float s[3], c[3];
 #pragma unroll
   for (int a = 0; a < 3; a++) {
@@ -242,7 +242,7 @@ __device__ __forceinline__ void encode_dir_fast(const float d[3], int n_freq_rt,
     __sincosf(d[a], &s[a], &c[a]);
   }
 #pragma unroll
-  for (int k = 0; k < n_freq; k++) {
+  for (int k = 0; k < NF; k++) {
 #pragma unroll
     for (int a = 0; a < 3; a++) {
       x[3 + 6 * k + a] = s[a];
@@ -254,36 +254,71 @@ __device__ __forceinline__ void encode_dir_fast(const float d[3], int n_freq_rt,
   }
 }
 
-template <typename T, int CC>
-__device__ __forceinline__ void tri_tile(const T* tile, int vb, int vx, int Cr, const int l[3], const float f[3],
-                                         float* out) {
-  const int C = CC ? CC : Cr;
+// The same with the channel and frequency counts known at run time only: the encoding and the 1 of
+// layer 1's folded bias, written into columns C .. C + 3 + 6 n_freq of row m of A (K = 144 layout), which
+// holds the features already.  Element by element: a row in registers cannot be indexed by C, and the
+// columns are the same for every thread, so their addresses cost next to nothing.
+constexpr int kMaxFreq = (kMaxIn - 3 - 1) / 6;  // C >= 1
+__device__ __forceinline__ void encode_dir_row(const float d[3], int C, int n_freq, char* act, int m) {
+  float e[3 + 6 * kMaxFreq];
+  encode_dir_fast<kMaxFreq>(d, e);
+  const int ne = 3 + 6 * n_freq;
+  char* row = act + tc::kmaj_off(m, 0, tc::kK2);
+  auto put = [&](int k, float v) {
+    *reinterpret_cast<__nv_bfloat16*>(row + (k >> 3) * 128 + (k & 7) * 2) = __float2bfloat16_rn(v);
+  };
+#pragma unroll
+  for (int j = 0; j < 3 + 6 * kMaxFreq; j++)
+    if (j < ne) put(C + j, e[j]);
+  if (C + ne < kMaxIn) put(C + ne, 1.0f);
+}
+
+// Four channels of a vertex of the staged brick or (GLOBAL) of the grid: a 16- or 8-byte load.
+template <bool GLOBAL>
+__device__ __forceinline__ float4 load4(const float* v) {
+  return GLOBAL ? __ldg(reinterpret_cast<const float4*>(v)) : *reinterpret_cast<const float4*>(v);
+}
+template <bool GLOBAL>
+__device__ __forceinline__ uint2 load4h(const __half* v) {
+  return GLOBAL ? __ldg(reinterpret_cast<const uint2*>(v)) : *reinterpret_cast<const uint2*>(v);
+}
+template <bool GLOBAL>
+__device__ __forceinline__ float4 load4(const __half* v) {
+  const uint2 a = load4h<GLOBAL>(v);
+  const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&a.x));
+  const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&a.y));
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
+// Trilinear interpolation of the features of a voxel into out[0, C), accumulated in FP32; at(x, y, z) is
+// its vertex (x, y, z in {0, 1}), in the staged brick or, GLOBAL, in the grid.  CC > 0
+// (a multiple of 4): four channels per load.  CC = 0: C <= kMaxC known at run time only; the loop over
+// channels is unrolled to the bound, so that out stays in registers.
+constexpr int kMaxC = 21;
+template <typename T, int CC, bool GLOBAL, typename At>
+__device__ __forceinline__ void tri_tile(At at, int C, const float f[3], float* out) {
+  constexpr int N = CC ? CC : kMaxC;
   const float fx = f[0], fy = f[1], fz = f[2];
-  for (int c = 0; c < C; c++) out[c] = 0.0f;
+#pragma unroll
+  for (int c = 0; c < N; c++) out[c] = 0.0f;
 #pragma unroll
   for (int q = 0; q < 8; q++) {
-    const int x = l[0] + (q & 1), y = l[1] + ((q >> 1) & 1), z = l[2] + (q >> 2);
     const float wq = ((q & 1) ? fx : 1.f - fx) * (((q >> 1) & 1) ? fy : 1.f - fy) * ((q >> 2) ? fz : 1.f - fz);
-    const T* v = tile + ((size_t)(z * vb + y) * vx + x) * C;
-    if constexpr (CC == 12 && sizeof(T) == 2) {
-      continue;  // handled by tri_tile_h2
-    } else if constexpr (CC == 12 && sizeof(T) == 4) {
-      const float4* v4 = reinterpret_cast<const float4*>(v);
+    const T* v = at(q & 1, (q >> 1) & 1, q >> 2);
+    if constexpr (CC > 0) {
+      static_assert(CC % 4 == 0, "four channels per load");
 #pragma unroll
-      for (int u = 0; u < 3; u++) {
-        float4 a = v4[u];
-        out[4 * u + 0] += wq * a.x;
-        out[4 * u + 1] += wq * a.y;
-        out[4 * u + 2] += wq * a.z;
-        out[4 * u + 3] += wq * a.w;
+      for (int u = 0; u < CC; u += 4) {
+        const float4 a = load4<GLOBAL>(v + u);
+        out[u + 0] += wq * a.x;
+        out[u + 1] += wq * a.y;
+        out[u + 2] += wq * a.z;
+        out[u + 3] += wq * a.w;
       }
     } else {
-      for (int c = 0; c < C; c++) {
-        float vv;
-        if constexpr (sizeof(T) == 4) vv = v[c];
-        else vv = __half2float(v[c]);
-        out[c] += wq * vv;
-      }
+#pragma unroll
+      for (int c = 0; c < N; c++)
+        if (c < C) out[c] += wq * (float)(GLOBAL ? __ldg(v + c) : v[c]);
     }
   }
 }
@@ -291,21 +326,20 @@ __device__ __forceinline__ void tri_tile(const T* tile, int vb, int vx, int Cr, 
 // FP16 grids, 12 channels: the eight corners accumulated in half2 (6 HFMA2 per corner).  The
 // accumulation error (~1e-3 worst case, features |f| <= 1) stays below the BF16 rounding of the
 // MLP input that follows.
-__device__ __forceinline__ void tri_tile_h2(const __half* tile, int vb, int vx, const int l[3], const float f[3],
-                                            float* out) {
+template <bool GLOBAL, typename At>
+__device__ __forceinline__ void tri_tile_h2(At at, const float f[3], float* out) {
   __half2 acc[6];
 #pragma unroll
   for (int u = 0; u < 6; u++) acc[u] = __float2half2_rn(0.0f);
   const float fx = f[0], fy = f[1], fz = f[2];
 #pragma unroll
   for (int q = 0; q < 8; q++) {
-    const int x = l[0] + (q & 1), y = l[1] + ((q >> 1) & 1), z = l[2] + (q >> 2);
     const float wq = ((q & 1) ? fx : 1.f - fx) * (((q >> 1) & 1) ? fy : 1.f - fy) * ((q >> 2) ? fz : 1.f - fz);
     const __half2 w2 = __float2half2_rn(wq);
-    const uint2* v2 = reinterpret_cast<const uint2*>(tile + ((size_t)(z * vb + y) * vx + x) * 12);
+    const __half* v = at(q & 1, (q >> 1) & 1, q >> 2);
 #pragma unroll
     for (int u = 0; u < 3; u++) {
-      uint2 a = v2[u];
+      uint2 a = load4h<GLOBAL>(v + 4 * u);
       acc[2 * u] = __hfma2(w2, *reinterpret_cast<__half2*>(&a.x), acc[2 * u]);
       acc[2 * u + 1] = __hfma2(w2, *reinterpret_cast<__half2*>(&a.y), acc[2 * u + 1]);
     }
@@ -422,15 +456,19 @@ __device__ __forceinline__ void hash_features(const HashGeo& h, const float p[3]
 // with alive false on entry it does nothing.
 // The grid's geometry `g` and the MLP dimensions are read where they live (kernel parameters for
 // one grid, the job table for a batch); `map` is the generic address of the feature grid's tensor map.
-// With HASH, the features come from the hash encoding `hg` instead of staged bricks (no TMA).
-template <typename T, int CC, int NF, bool HASH = false>
+// SRC: where the features come from.  Staged: the tile's brick, copied into shared memory by TMA.
+// Direct: the grid `feat` in global memory.  Hash: the hash encoding `hg`.
+enum class Src { Staged, Direct, Hash };
+template <typename T, int CC, int NF, Src SRC>
 __device__ __forceinline__ bool gather_tiles(char* sm, tc::Group& G, const GridGeo& g, const CUtensorMap* map,
                                              int in_dim, int n_freq, int vb, int vx, int box_bytes, const RenderWs& w,
                                              long long t_begin, long long t_end, int& loaded, bool alive,
-                                             const HashGeo* hg = nullptr) {
+                                             const T* feat, const HashGeo* hg = nullptr) {
   using namespace tc;
+  constexpr bool HASH = SRC == Src::Hash, STAGED = SRC == Src::Staged;
   if (!alive) return false;
-  const int B = g.brick, C = CC ? CC : g.C, m = G.m;
+  // features of a sample: 2 per level of a hash encoding, else the grid's channels
+  const int B = g.brick, C = CC ? CC : (HASH ? in_dim - 3 - 6 * n_freq : g.C), m = G.m;
   const T* tile = (const T*)G.tile;
   // Tile descriptors run two tiles ahead of the gather and record payloads one tile ahead, and a
   // payload load is never conditional on loaded data (rows past a tile's count re-read its last
@@ -466,7 +504,7 @@ __device__ __forceinline__ bool gather_tiles(char* sm, tc::Group& G, const GridG
     osid = kNoRecord;
   };
   bool tma_pending = false, mma_pending = false;
-  if (!HASH && t_begin < t_end) {
+  if (STAGED && t_begin < t_end) {
     if (m == 0) tma_brick(tg);
     loaded = (int)tg.z;
     tma_pending = true;
@@ -487,7 +525,7 @@ __device__ __forceinline__ bool gather_tiles(char* sm, tc::Group& G, const GridG
       }
       mma_pending = true;
       // every thread is done with the staged brick: copy the next tile's brick if it differs
-      if (!HASH && gather && (int)tg.z != loaded) {
+      if (STAGED && gather && (int)tg.z != loaded) {
         if (m == 0) tma_brick(tg);
         loaded = (int)tg.z;
         tma_pending = true;
@@ -551,17 +589,35 @@ __device__ __forceinline__ bool gather_tiles(char* sm, tc::Group& G, const GridG
           }
           if (!ok)
             set_err(&w.hdr[0], kErrInternal);
-          else if constexpr (CC == 12 && sizeof(T) == 2)
-            tri_tile_h2((const __half*)tile, vb, vx, l, f, x);
-          else
-            tri_tile<T, CC>(tile, vb, vx, C, l, f, x);
+          else {
+            auto tri = [&](auto at) {
+              if constexpr (CC == 12 && sizeof(T) == 2) tri_tile_h2<!STAGED>(at, f, x);
+              else tri_tile<T, CC, !STAGED>(at, C, f, x);
+            };
+            if constexpr (STAGED) {
+              tri([&](int cx, int cy, int cz) {
+                return tile + ((size_t)((l[2] + cz) * vb + l[1] + cy) * vx + l[0] + cx) * C;
+              });
+            } else {
+              const size_t sy = (size_t)g.n[0] * C, sz = sy * g.n[1];
+              const T* v0 = feat + (size_t)(l[2] + bz * B) * sz + (size_t)(l[1] + by * B) * sy +
+                            (size_t)(l[0] + bx * B) * C;
+              tri([&](int cx, int cy, int cz) { return v0 + cz * sz + cy * sy + cx * C; });
+            }
+          }
         }
-        const float d[3] = {gdir.y, gdir.z, gdir.w};
-        encode_dir_fast<NF>(d, n_freq, x + C);
-        if (in_dim < kK1) x[CC && NF ? (CC + 3 + 6 * NF) % kK1 : in_dim % kK1] = 1.0f;  // folded layer-1 bias
+        if constexpr (CC > 0 && NF > 0) {
+          const float d[3] = {gdir.y, gdir.z, gdir.w};
+          encode_dir_fast<NF>(d, x + CC);
+          if (CC + 3 + 6 * NF < kK1) x[(CC + 3 + 6 * NF) % kK1] = 1.0f;  // folded layer-1 bias
+        }
       }
 #pragma unroll
       for (int k0 = 0; k0 < kK1; k0 += 8) store_chunk(G.act, m, k0, kK2, x + k0);
+      if constexpr (CC == 0 || NF == 0) {
+        const float d[3] = {gdir.y, gdir.z, gdir.w};
+        if (m < mcnt) encode_dir_row(d, C, n_freq, G.act, m);
+      }
       fence_proxy_async();
     }
     if (run) {
@@ -595,10 +651,11 @@ __device__ __forceinline__ bool gather_tiles(char* sm, tc::Group& G, const GridG
 
 // The persistent gather + MLP kernel of the BF16 path for one grid (launched with 128 * groups
 // threads): each CTA takes a contiguous range of tiles, split evenly among its groups.
-template <typename T, int CC, int NF>
-__global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16(GridGeo g, int S, MlpPtrs mlp, RenderWs w,
-                                                            const __grid_constant__ CUtensorMap fmap, int vb, int vx,
-                                                            int box_bytes, int groups) {
+template <typename T, int CC, int NF, Src SRC>
+__global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16(GridGeo g, MlpPtrs mlp, RenderWs w,
+                                                            const __grid_constant__ CUtensorMap fmap,
+                                                            const T* __restrict__ feat, int vb, int vx, int box_bytes,
+                                                            int groups) {
   using namespace tc;
   extern __shared__ __align__(1024) char sm[];
   Group G = setup(sm, &mlp, groups, box_bytes);
@@ -609,7 +666,8 @@ __global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16(GridGeo g, int S, Ml
   const uint32_t span = c_end > c_begin ? c_end - c_begin : 0;
   const long long t_begin = c_begin + (span * G.g) / groups, t_end = c_begin + (span * (G.g + 1)) / groups;
   int loaded = -1;
-  gather_tiles<T, CC, NF>(sm, G, g, &fmap, mlp.in_dim, mlp.n_freq, vb, vx, box_bytes, w, t_begin, t_end, loaded, true);
+  gather_tiles<T, CC, NF, SRC>(sm, G, g, &fmap, mlp.in_dim, mlp.n_freq, vb, vx, box_bytes, w, t_begin, t_end, loaded,
+                               true, feat);
   tmem_free_all(tmem_base);
 }
 
@@ -628,8 +686,8 @@ __global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16_hash(GridGeo g, MlpP
   const uint32_t span = c_end > c_begin ? c_end - c_begin : 0;
   const long long t_begin = c_begin + (span * G.g) / groups, t_end = c_begin + (span * (G.g + 1)) / groups;
   int loaded = -1;
-  gather_tiles<T, CC, NF, true>(sm, G, g, nullptr, mlp.in_dim, mlp.n_freq, 0, 0, 0, w, t_begin, t_end, loaded, true,
-                                &hg);
+  gather_tiles<T, CC, NF, Src::Hash>(sm, G, g, nullptr, mlp.in_dim, mlp.n_freq, 0, 0, 0, w, t_begin, t_end, loaded,
+                                     true, nullptr, &hg);
   tmem_free_all(tmem_base);
 }
 
@@ -638,7 +696,7 @@ __global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16_hash(GridGeo g, MlpP
 // tiles, split evenly among its groups, as a launch per job would; so at any moment the GPU works on
 // one or two jobs' grids, which keeps their bricks in L2.  The CTA stages each job's geometry in
 // shared memory and loads the job's MLP weights when they differ from the ones there.
-template <typename T, int CC, int NF>
+template <typename T, int CC, int NF, Src SRC>
 __global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16_batch(const JobDesc* __restrict__ jobs, int n_jobs,
                                                                   RenderWs w, int vb, int vx, int box_bytes,
                                                                   int groups) {
@@ -666,8 +724,8 @@ __global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16_batch(const JobDesc*
     __syncthreads();
     const long long span = b - a;
     const long long t0 = a + (span * G.g) / groups, t1 = a + (span * (G.g + 1)) / groups;
-    alive = gather_tiles<T, CC, NF>(sm, G, geo, &J.map, J.mlp.in_dim, J.mlp.n_freq, vb, vx, box_bytes, w, t0, t1,
-                                    loaded, alive);
+    alive = gather_tiles<T, CC, NF, SRC>(sm, G, geo, &J.map, J.mlp.in_dim, J.mlp.n_freq, vb, vx, box_bytes, w, t0, t1,
+                                         loaded, alive, (const T*)J.features);
   }
   tmem_free_all(tmem_base);
 }
@@ -703,28 +761,55 @@ __global__ void __launch_bounds__(512, 1) k_mlp_eval_bf16(MlpPtrs mlp, const flo
 
 // -------------------------------------------------------------------------------------------
 
-// Tile pipelines per CTA: as many as fit the shared memory, at most `requested` (0 = no limit).
-static int tc_groups(int box_bytes, int requested) {
+// Tile pipelines per CTA (at most `requested`, 0 = no limit) and where they take the features from;
+// 0 when not even one staged brick fits the shared memory.  Where the staged bricks leave room for two
+// pipelines at most, four that read the features from global memory are faster, since the kernel is
+// bound by the latency of each tile's chain: 18.4 M samples of a 96 x 113 x 80 FP32 grid, bricks of 8,
+// 1481 -> 1121 us with 8 channels and 1580 -> 1313 us with 12.  At three the copies win on large grids
+// (62.5 M samples of a 256^3 x 12 FP16 grid: 3660 staged, 3782 us direct), at four everywhere.
+constexpr int kStagedGroups = 3;
+static int tc_groups(int box_bytes, int requested, bool* direct) {
   using namespace tc;
   int groups = kMaxGroups;
-  while (groups > 1 && Smem::groups + groups * group_bytes(box_bytes) > 227 * 1024) groups--;
+  while (groups > 0 && Smem::groups + groups * group_bytes(box_bytes) > 227 * 1024) groups--;
+  *direct = groups > 0 && groups < kStagedGroups && (requested == 0 || requested > groups);
+  if (groups == 0) return 0;
+  if (*direct) groups = kMaxGroups;
   return requested > 0 && requested < groups ? requested : groups;
 }
 
-template <typename T, int CC, int NF>
-static cicero_status launch_tc(const GridGeo& geo, int S, const MlpPtrs& mlp, const RenderWs& ws,
-                               const CUtensorMap& map, const BrickBox& box, int mlp_groups, cudaStream_t st) {
+// Calls go<C, n_freq> with the channel count and the frequencies as constants where they are specialised
+// (4, 8, 12 or 16 channels with 4 frequencies), else with zeros.  The specialised kernels load four
+// channels at a time and keep the input row in registers: 8 channels of an FP32 grid, 18.4 M samples,
+// bricks of 4: 2091 us with the row indexed at run time, 924 us specialised.
+template <typename F>
+static cicero_status by_channels(int C, int n_freq, F go) {
+  using std::integral_constant;
+  constexpr integral_constant<int, 0> any;
+  constexpr integral_constant<int, 4> four;
+  if (n_freq != 4) return go(any, any);
+  switch (C) {
+    case 4: return go(four, four);
+    case 8: return go(integral_constant<int, 8>(), four);
+    case 12: return go(integral_constant<int, 12>(), four);
+    case 16: return go(integral_constant<int, 16>(), four);
+    default: return go(any, any);
+  }
+}
+
+template <typename T, int CC, int NF, Src SRC>
+static cicero_status launch_tc(const GridGeo& geo, const MlpPtrs& mlp, const RenderWs& ws, const CUtensorMap& map,
+                               const void* feat, const BrickBox& box, int groups, cudaStream_t st) {
   using namespace tc;
-  const int groups = tc_groups(box.box_bytes, mlp_groups);
-  int smem = Smem::groups + groups * group_bytes(box.box_bytes);
-  if (smem > 227 * 1024) return fail(CICERO_ERR_UNSUPPORTED, "brick too large for the tensor-core kernel");
-  smem = std::max(smem, 120 * 1024);  // one CTA per SM: it owns all 512 TMEM columns
-  auto kern = k_gather_mlp_bf16<T, CC, NF>;
+  const int box_bytes = SRC == Src::Staged ? box.box_bytes : 0;
+  const int smem = std::max(Smem::groups + groups * group_bytes(box_bytes), 120 * 1024);  // one CTA per SM: it owns
+                                                                                           // all 512 TMEM columns
+  auto kern = k_gather_mlp_bf16<T, CC, NF, SRC>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_gather_mlp_bf16)");
   {
     ProfScope ps(kStGatherMlp, st);
-    kern<<<num_sms(), 128 * groups, smem, st>>>(geo, S, mlp, ws, map, box.vb, box.vx, box.box_bytes, groups);
+    kern<<<num_sms(), 128 * groups, smem, st>>>(geo, mlp, ws, map, (const T*)feat, box.vb, box.vx, box_bytes, groups);
   }
   count_launches(1);
   e = cudaGetLastError();
@@ -735,11 +820,19 @@ cicero_status launch_gather_mlp_bf16(const cicero_grid* grid, const GridGeo& geo
                                      const MlpPtrs& mlp, const RenderWs& ws, const CUtensorMap& map,
                                      const BrickBox& box, cudaStream_t st) {
   const bool f16 = grid->dtype == CICERO_F16;
-  if (geo.C == 12 && mlp.n_freq == 4)
-    return f16 ? launch_tc<__half, 12, 4>(geo, ws.S, mlp, ws, map, box, mlp_groups, st)
-               : launch_tc<float, 12, 4>(geo, ws.S, mlp, ws, map, box, mlp_groups, st);
-  return f16 ? launch_tc<__half, 0, 0>(geo, ws.S, mlp, ws, map, box, mlp_groups, st)
-             : launch_tc<float, 0, 0>(geo, ws.S, mlp, ws, map, box, mlp_groups, st);
+  // the specialised channel counts (vector loads, the input row laid out at compile time) and the rest
+  bool direct;
+  const int groups = tc_groups(box.box_bytes, mlp_groups, &direct);
+  if (groups == 0) return fail(CICERO_ERR_UNSUPPORTED, "brick too large for the tensor-core kernel");
+  return by_channels(geo.C, mlp.n_freq, [&](auto cc, auto nf) {
+    constexpr int CC = decltype(cc)::value, NF = decltype(nf)::value;
+    const void* feat = grid->features;
+    if (direct)
+      return f16 ? launch_tc<__half, CC, NF, Src::Direct>(geo, mlp, ws, map, feat, box, groups, st)
+                 : launch_tc<float, CC, NF, Src::Direct>(geo, mlp, ws, map, feat, box, groups, st);
+    return f16 ? launch_tc<__half, CC, NF, Src::Staged>(geo, mlp, ws, map, feat, box, groups, st)
+               : launch_tc<float, CC, NF, Src::Staged>(geo, mlp, ws, map, feat, box, groups, st);
+  });
 }
 
 template <typename T, int CC, int NF>
@@ -768,14 +861,12 @@ cicero_status launch_gather_mlp_bf16_hash(const GridGeo& geo, const MlpPtrs& mlp
   return hg.f16 ? launch_tc_hash<__half, 0, 0>(geo, mlp, ws, hg, st) : launch_tc_hash<float, 0, 0>(geo, mlp, ws, hg, st);
 }
 
-template <typename T, int CC, int NF>
-static cicero_status launch_tc_batch(const BatchPlan& b, cudaStream_t st) {
+template <typename T, int CC, int NF, Src SRC>
+static cicero_status launch_tc_batch(const BatchPlan& b, int groups, cudaStream_t st) {
   using namespace tc;
-  const int groups = tc_groups(b.box.box_bytes, b.mlp_groups);
-  int smem = Smem::groups + groups * group_bytes(b.box.box_bytes);
-  if (smem > 227 * 1024) return fail(CICERO_ERR_UNSUPPORTED, "brick too large for the tensor-core kernel");
-  smem = std::max(smem, 120 * 1024);  // one CTA per SM: it owns all 512 TMEM columns
-  auto kern = k_gather_mlp_bf16_batch<T, CC, NF>;
+  const int box_bytes = SRC == Src::Staged ? b.box.box_bytes : 0;
+  const int smem = std::max(Smem::groups + groups * group_bytes(box_bytes), 120 * 1024);  // as in launch_tc
+  auto kern = k_gather_mlp_bf16_batch<T, CC, NF, SRC>;
   // set once per size, so that a launch after the first one is pure kernel launches (graph capture)
   static std::atomic<int> smem_set{0};
   cudaError_t e = cudaSuccess;
@@ -786,7 +877,7 @@ static cicero_status launch_tc_batch(const BatchPlan& b, cudaStream_t st) {
   }
   {
     ProfScope ps(kStGatherMlp, st);
-    kern<<<num_sms(), 128 * groups, smem, st>>>(b.jobs, b.n_jobs, b.ws, b.box.vb, b.box.vx, b.box.box_bytes, groups);
+    kern<<<num_sms(), 128 * groups, smem, st>>>(b.jobs, b.n_jobs, b.ws, b.box.vb, b.box.vx, box_bytes, groups);
   }
   count_launches(1);
   e = cudaGetLastError();
@@ -794,9 +885,17 @@ static cicero_status launch_tc_batch(const BatchPlan& b, cudaStream_t st) {
 }
 
 cicero_status launch_gather_mlp_bf16_batch(const BatchPlan& b, cudaStream_t st) {
-  if (b.C == 12 && b.n_freq == 4)
-    return b.f16 ? launch_tc_batch<__half, 12, 4>(b, st) : launch_tc_batch<float, 12, 4>(b, st);
-  return b.f16 ? launch_tc_batch<__half, 0, 0>(b, st) : launch_tc_batch<float, 0, 0>(b, st);
+  bool direct;
+  const int groups = tc_groups(b.box.box_bytes, b.mlp_groups, &direct);
+  if (groups == 0) return fail(CICERO_ERR_UNSUPPORTED, "brick too large for the tensor-core kernel");
+  return by_channels(b.C, b.n_freq, [&](auto cc, auto nf) {
+    constexpr int CC = decltype(cc)::value, NF = decltype(nf)::value;
+    if (direct)
+      return b.f16 ? launch_tc_batch<__half, CC, NF, Src::Direct>(b, groups, st)
+                   : launch_tc_batch<float, CC, NF, Src::Direct>(b, groups, st);
+    return b.f16 ? launch_tc_batch<__half, CC, NF, Src::Staged>(b, groups, st)
+                 : launch_tc_batch<float, CC, NF, Src::Staged>(b, groups, st);
+  });
 }
 
 cicero_status launch_mlp_eval_bf16(const MlpPtrs& mlp, const float* x, int M, float* c, uint32_t* err,
