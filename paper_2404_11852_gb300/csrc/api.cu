@@ -716,8 +716,8 @@ size_t cicero_warp_workspace_size(const cicero_camera* tgt_cam) {
 
 // The backward's plan: FP32, bricks of 16 up to 16 channels (the tensor-core kernels and the
 // CUDA-core weight-gradient kernel read features from global memory, so a brick only groups the
-// samples: larger bricks give fewer, fuller 128-sample tiles); bricks of 4 above that, where the
-// FP32 recompute stages each brick in shared memory beside its two input buffers.
+// samples: larger bricks give fewer, fuller 128-sample tiles); bricks of 4 above that, a box that an
+// FP32 render takes for every channel count.
 static cicero_options backward_options(const cicero_grid* grid) {
   cicero_options o;
   memset(&o, 0, sizeof o);

@@ -220,6 +220,11 @@ cicero_status launch_gather_mlp_bf16(const cicero_grid* grid, const GridGeo& geo
 cicero_status launch_mlp_eval_bf16(const MlpPtrs& mlp, const float* x, int M, float* c, uint32_t* err,
                                    cudaStream_t st);
 
+// FP32-class Feature Gathering + Computation on the tensor cores, operands split into 2 or 3 BF16 parts
+// (mlp_split.cu)
+cicero_status launch_mlp_split(const cicero_grid* grid, const GridGeo& geo, int parts, const MlpPtrs& mlp,
+                               const RenderWs& ws, cudaStream_t st);
+
 // SpaRW warp (warp.cu)
 struct WarpArgs {
   int wr, hr;          // reference image

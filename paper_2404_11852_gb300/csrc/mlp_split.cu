@@ -1,0 +1,610 @@
+// Feature Gathering + Feature Computation with FP32-class accuracy on the tensor cores (tcgen05,
+// sm_103a): operands split into BF16 parts, products accumulated in FP32 in tensor memory.
+//
+//   NP = 3  v = hi + mid + lo (24 significant bits), the six products above 2^-24: FP32 accuracy
+//   NP = 2  v = hi + lo (16 bits), three products (Henry, Tang and Heinecke, ARITH 2019)
+//
+// One persistent CTA per SM, a pipeline of roles over the CTA's tiles of 128 samples of one brick:
+//   G   two groups of 4 warps (alternate tiles), a thread per sample: interpolates the features from
+//       global memory, encodes the direction, splits the input row into operand x (shared memory)
+//   M   one thread: issues every MMA.  Layer 1: D = x W1^T, both operands in shared memory.
+//       Layer 2: D = h1 W2^T with h1 read from tensor memory, in two chunks of 64 hidden units
+//   E1  8 warps, two threads per sample (half of the hidden units each): layer 1's accumulators ->
+//       bias, ReLU, split -> h1 in tensor memory, chunk by chunk
+//   E2  8 warps: layer 2's accumulators -> bias, ReLU, layer 3 in FP32, sigmoid -> (c, w) into the
+//       sample's record
+// Layer 1 of tile i + 1 is issued between the two chunks of layer 2 of tile i, and h1's chunk c of tile
+// i + 1 is written as soon as chunk c of tile i has been read, so the tensor pipe runs on while E1 and
+// E2 work.
+// Order of the products: a tensor-core accumulation rounds its running sum towards zero, so the more
+// steps are added to a sum of full size, the further it drifts.  The hi hi products come last, after all
+// the small ones of both chunks: 8 steps at full size in layer 2 instead of 48.  The hi part of h1
+// then outlives the others, hence its two buffers.
+//
+// What bounds it: with NP = 3 the MMAs, (48 + 128) / 16 K steps x 6 products of M = N = 128 at 64 clocks
+// each, 4,224 clocks a tile of the ~5,000 measured.  With h1 in tensor memory layer 2 reads one operand
+// from shared memory, half of what a tile of two shared operands needs.  With NP = 2 (2,112 clocks of
+// MMAs, ~3,900 measured) the latency of G's and E1's instructions.
+// Measured, gather + MLP: 62.5 M samples of a 256^3 x 12 FP16 grid, NP = 3, 52.5 ms on the CUDA cores
+// before, 8.7 ms; 6.7 M samples of a 160^3 x 12 FP16 grid, NP = 2, 1.70 ms (one thread per sample for
+// everything, two tiles in flight) before, 0.70 ms.  Steps on the way: E1 and E2 as one role 12.0 / 0.93
+// ms; the MMAs issued with warp-uniform operands 13.4 -> 9.8; h1 in two chunks instead of four 10.4 -> 8.9.
+// All waits are bounded; a role that runs into a timeout records it and leaves, and so do the others.
+#include <cuda_runtime.h>
+
+#include "common.cuh"
+#include "internal.h"
+#include "tc_ptx.cuh"
+
+namespace cicero {
+
+namespace ms {
+
+constexpr int kK1 = kMaxIn;                 // layer-1 K: the input row padded to 48
+constexpr int kEpiWarps = 8, kGatWarps = 4;  // warps of E1 and of E2; warps of one of G's two groups
+constexpr int kE2 = kEpiWarps, kG = 2 * kEpiWarps, kM = kG + 2 * kGatWarps;  // first warp of each role
+constexpr int kThreads = 32 * (kM + 4);      // M's warpgroup has one working warp
+// Registers per thread: 72 at launch (28 warps), then shared out by role (setmaxnreg):
+// 256 (88 + 80 + 72) + 128 x 24 = 896 x 72.
+constexpr int kRegsE1 = 88, kRegsE2 = 80, kRegsG = 72, kRegsM = 24;
+static_assert(kThreads == 896 && 256 * (kRegsE1 + kRegsE2 + kRegsG) + 128 * kRegsM <= kThreads * 72, "register shares");
+template <int R>
+__device__ __forceinline__ void regs_up() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R));
+}
+template <int R>
+__device__ __forceinline__ void regs_down() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R));
+}
+constexpr int kChunks = 2;                  // chunks of hidden units of layer 2's K
+constexpr int kMeta = 4;                    // tiles of per-sample data in flight
+constexpr int kXBytes = kTile * kK1 * 2;    // one part of the input operand
+constexpr int kW1Bytes = kHidden * kK1 * 2, kW2Bytes = kHidden * kHidden * 2;
+
+template <int NP>
+struct Smem {
+  static constexpr int w1 = 0;                               // [NP][128][48] bf16: row n, K = k: W1[n][k]
+  static constexpr int w2 = w1 + NP * kW1Bytes;              // [NP][128][128]
+  static constexpr int x = w2 + NP * kW2Bytes;               // [2][NP][128][48]: the input rows of two tiles
+  static constexpr int b1 = x + 2 * NP * kXBytes;            // [128] f32
+  static constexpr int l3 = b1 + kHidden * 4;                // per pair of hidden units: b2, w3 rows 0, 1, 2
+  static constexpr int b3 = l3 + 4 * kHidden * 4;            // [4]
+  static constexpr int z = b3 + 16;                          // [kMeta][128] float4: partial layer-3 sums
+  static constexpr int meta = z + kMeta * kTile * 16;        // [kMeta][128] float4: record, weight
+  static constexpr int bars = meta + kMeta * kTile * 16;
+  static constexpr int bytes = bars + 8 * 32;
+  static_assert(x % 16 == 0 && w2 % 16 == 0 && bars % 16 == 0 && bytes <= 227 * 1024, "layout");
+};
+
+struct Bars {  // one phase per use, in tile order
+  uint64_t xfull[2];       // x of tile i written                          (4 G warps)
+  uint64_t l1done[2];      // layer 1 of tile i done, x free               (commit)
+  uint64_t afull[kChunks]; // chunk c of h1 written                        (8 E1 warps)
+  uint64_t cdone[kChunks]; // chunk c of h1 but its hi part read           (commit)
+  uint64_t l2done[2];      // layer 2 of tile i done                       (commit)
+  uint64_t dfree[2];       // accumulator of tile i read                   (8 E2 warps)
+  uint64_t zfull[kMeta];   // partial layer-3 sums of tile i written       (4 E2 warps)
+  uint64_t mfull[kMeta];   // per-sample data of tile i written            (4 G warps)
+  uint64_t last;           // every MMA done                               (commit)
+  uint32_t tmem;
+};
+static_assert(sizeof(Bars) <= 8 * 32, "barrier block");
+
+__device__ __forceinline__ void arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// after every lane's writes (and its fence): one arrival per warp
+__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) arrive(bar);
+}
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, uint32_t* err) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
+}
+
+// Columns 32 c + 16 h + j (c < 4, j < 16) of this thread's lane of the accumulator at d, into v[16 c + j].
+__device__ __forceinline__ void load_half(uint32_t d, int h, float* v) {
+  uint32_t r[64];
+  const uint32_t a = d + 16u * (uint32_t)h;
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%64];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%65];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47}, [%66];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%67];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]),
+        "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]),
+        "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]),
+        "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]),
+        "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+      : "r"(a), "r"(a + 32u), "r"(a + 64u), "r"(a + 96u)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 64; i++) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+
+// two packed FP32 operations
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 p, q, s;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tadd.rn.f32x2 s, p, q;\n\t"
+      "mov.b64 {%0, %1}, s;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 r;
+  asm("{\n\t.reg .b64 p, q, t, s;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tmov.b64 t, {%6, %7};\n\t"
+      "fma.rn.f32x2 s, p, q, t;\n\tmov.b64 {%0, %1}, s;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
+}
+
+// (a, b) split into NP packed BF16 parts: each part rounds what the ones before it left.
+template <int NP>
+__device__ __forceinline__ void split2(float2 v, uint32_t p[NP]) {
+#pragma unroll
+  for (int k = 0; k < NP; k++) {
+    p[k] = tc::pack_bf16(v.x, v.y);
+    if (k + 1 < NP)  // v - part, exactly
+      v = fma2(make_float2(__uint_as_float(p[k] << 16), __uint_as_float(p[k] & 0xffff0000u)),
+               make_float2(-1.0f, -1.0f), v);
+  }
+}
+
+// The NP operand rows (16 bytes each) of 8 consecutive K values of one row.
+template <int NP>
+__device__ __forceinline__ void split_row(const float* v, uint4 q[NP]) {
+  uint32_t p[4][NP];
+#pragma unroll
+  for (int j = 0; j < 4; j++) split2<NP>(make_float2(v[2 * j], v[2 * j + 1]), p[j]);
+#pragma unroll
+  for (int k = 0; k < NP; k++) q[k] = make_uint4(p[0][k], p[1][k], p[2][k], p[3][k]);
+}
+
+// The products of one K step of 16 but the largest (hi hi): those of parts a + b < NP, smallest first.
+template <int NP, typename MMA>
+__device__ __forceinline__ void small_products(MMA mma) {
+#pragma unroll
+  for (int s = NP - 1; s > 0; s--)
+#pragma unroll
+    for (int a = 0; a <= s; a++) mma(a, s - a);
+}
+
+// Tensor memory: part k of h1 of tile i at h1_col (two buffers of the hi part), then the accumulators.
+template <int NP>
+struct Tmem {
+  static constexpr uint32_t acc = 64 * (NP + 1);  // accumulator of tile i: + 128 (i & 1)
+  static_assert(acc + 256 <= 512, "tensor memory");
+};
+__device__ __forceinline__ uint32_t h1_col(int k, uint32_t i) { return k == 0 ? 64u * (i & 1) : 64u * (uint32_t)(k + 1); }
+
+// Weights [rows][in] (FP32, global) into NP K-major operands of K columns (zeros from `in` on).
+template <int NP>
+__device__ __forceinline__ void load_weights(char* dst, int part_bytes, const float* w, int rows, int in, int K) {
+  const int chunks = rows * (K / 8);
+  const bool vec = (in & 3) == 0 && (reinterpret_cast<uintptr_t>(w) & 15u) == 0;
+#pragma unroll 2
+  for (int i = threadIdx.x; i < chunks; i += kThreads) {
+    const int n = i / (K / 8), k0 = (i % (K / 8)) * 8;
+    const float* src = w + (size_t)n * in + k0;
+    float v[8];
+    if (vec && k0 + 8 <= in) {
+      const float4 a = __ldg(reinterpret_cast<const float4*>(src)), b = __ldg(reinterpret_cast<const float4*>(src) + 1);
+      v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; j++) v[j] = k0 + j < in ? __ldg(src + j) : 0.0f;
+    }
+    uint4 q[NP];
+    split_row<NP>(v, q);
+#pragma unroll
+    for (int p = 0; p < NP; p++) *reinterpret_cast<uint4*>(dst + p * part_bytes + tc::kmaj_off(n, k0, K)) = q[p];
+  }
+}
+
+__device__ __forceinline__ float4 ld4(const float* v) { return __ldg(reinterpret_cast<const float4*>(v)); }
+__device__ __forceinline__ float4 ld4(const __half* v) {
+  const uint2 a = __ldg(reinterpret_cast<const uint2*>(v));
+  const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&a.x));
+  const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&a.y));
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
+constexpr int kMaxC = 21;
+// Trilinear features of voxel i0 at fractions f, from global memory, into out[0, C) (FP32; the rest of
+// out untouched).  CC > 0: C = CC.
+template <typename T, int CC>
+__device__ __forceinline__ void gather(const GridGeo& g, const T* __restrict__ feat, const int i0[3], const float f[3],
+                                       float* out) {
+  const int C = CC ? CC : g.C;
+  constexpr int N = CC ? CC : kMaxC;
+#pragma unroll
+  for (int q = 0; q < 8; q++) {
+    const float wq = ((q & 1) ? f[0] : 1.f - f[0]) * (((q >> 1) & 1) ? f[1] : 1.f - f[1]) * ((q >> 2) ? f[2] : 1.f - f[2]);
+    const T* v = feat + (((size_t)(i0[2] + (q >> 2)) * g.n[1] + (i0[1] + ((q >> 1) & 1))) * g.n[0] + (i0[0] + (q & 1))) * C;
+    if (CC ? CC % 4 == 0 : (C & 3) == 0) {  // rows of the grid start on 16 bytes, vertices on 4 channels
+#pragma unroll
+      for (int c = 0; c + 4 <= N; c += 4)
+        if (CC || c < C) {
+          const float4 a = ld4(v + c);
+          out[c] = fmaf(wq, a.x, out[c]);
+          out[c + 1] = fmaf(wq, a.y, out[c + 1]);
+          out[c + 2] = fmaf(wq, a.z, out[c + 2]);
+          out[c + 3] = fmaf(wq, a.w, out[c + 3]);
+        }
+    } else {
+#pragma unroll
+      for (int c = 0; c < N; c++)
+        if (c < C) out[c] = fmaf(wq, ldf(v + c), out[c]);
+    }
+  }
+}
+
+// d, then sin/cos(2^k d) for k < NF (the recurrence of encode_dir), unrolled
+template <int NF>
+__device__ __forceinline__ void encode(const float d[3], float* x) {
+  float s[3], c[3];
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    x[a] = d[a];
+    sincosf(d[a], &s[a], &c[a]);
+  }
+#pragma unroll
+  for (int k = 0; k < NF; k++) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      x[3 + 6 * k + a] = s[a];
+      x[3 + 6 * k + 3 + a] = c[a];
+      const float s2 = 2.0f * s[a] * c[a];
+      c[a] = 1.0f - 2.0f * s[a] * s[a];
+      s[a] = s2;
+    }
+  }
+}
+
+// M: every MMA of the CTA's n tiles, by one warp: the control flow and the operands are the warp's, one
+// elected lane issues.  (Issued from a thread of its own, each MMA's operands took a dozen instructions
+// through per-thread registers: ~110 clocks an MMA beside 27 other warps, against the 64 it runs.)
+template <int NP>
+__device__ __forceinline__ void issue_mmas(char* sm, Bars& B, uint32_t tmem, uint32_t n, uint32_t* err) {
+  using namespace tc;
+  using S = Smem<NP>;
+  tmem = __shfl_sync(0xffffffffu, tmem, 0);
+  n = __shfl_sync(0xffffffffu, n, 0);
+  const uint32_t dcol = tmem + Tmem<NP>::acc;
+  constexpr uint32_t hi1 = desc_hi(kK1 * 16), hi2 = desc_hi(kHidden * 16), id = idesc_bf16(kHidden);
+  const uint32_t x = desc_lo(smem_u32(sm + S::x), 128u);
+  const uint32_t w1 = desc_lo(smem_u32(sm + S::w1), 128u);
+  const uint32_t w2 = desc_lo(smem_u32(sm + S::w2), 128u);
+  const bool leader = elect_one();
+  auto layer1 = [&](uint32_t i) -> bool {
+    if (!warp_wait(&B.xfull[i & 1], (i >> 1) & 1, err)) return false;
+    if (i >= 2 && !warp_wait(&B.dfree[i & 1], ((i >> 1) - 1) & 1, err)) return false;
+    fence_after();
+    const uint32_t d = dcol + 128u * (i & 1);
+    const uint32_t xo = x + (i & 1) * (NP * kXBytes / 16);
+    if (leader) {
+#pragma unroll
+      for (int s = 0; s < kK1 / 16; s++)
+        small_products<NP>([&](int a, int b) {
+          mma_u<hi1, hi1, id>(d, xo + (a * (kXBytes / 16) + 16 * s), w1 + (b * (kW1Bytes / 16) + 16 * s),
+                              (s > 0 || a > 0 || b < NP - 1) ? 1u : 0u);
+        });
+#pragma unroll
+      for (int s = 0; s < kK1 / 16; s++) mma_u<hi1, hi1, id>(d, xo + 16 * s, w1 + 16 * s, 1u);
+      mma_commit(&B.l1done[i & 1]);
+    }
+    __syncwarp();
+    return true;
+  };
+  bool alive = layer1(0);
+  for (uint32_t i = 0; i < n && alive; i++) {
+    const uint32_t d = dcol + 128u * (i & 1);
+#pragma unroll
+    for (int c = 0; c < kChunks; c++) {
+      if (c == kChunks / 2 && i + 1 < n && !(alive = layer1(i + 1))) break;
+      if (!(alive = warp_wait(&B.afull[c], i & 1, err))) break;
+      fence_after();
+      if (leader) {
+#pragma unroll
+        for (int s = c * (8 / kChunks); s < (c + 1) * (8 / kChunks); s++)
+          small_products<NP>([&](int a, int b) {
+            mma_u_ta<hi2, id>(d, tmem + h1_col(a, i) + 8u * s, w2 + (b * (kW2Bytes / 16) + 16 * s),
+                              (s > 0 || a > 0 || b < NP - 1) ? 1u : 0u);
+          });
+        mma_commit(&B.cdone[c]);
+        if (c == kChunks - 1) {
+#pragma unroll
+          for (int s = 0; s < kHidden / 16; s++) mma_u_ta<hi2, id>(d, tmem + h1_col(0, i) + 8u * s, w2 + 16 * s, 1u);
+          mma_commit(&B.l2done[i & 1]);
+        }
+      }
+      __syncwarp();
+    }
+  }
+  if (leader) {
+    mma_commit(&B.last);
+    mbar_wait(&B.last, 0, err);  // nothing in flight when tensor memory is given back
+  }
+  __syncwarp();
+}
+
+// CC, NF: channels and frequencies as constants (12 and 4), or 0: known at run time only.
+template <int NP, int CC, int NF>
+__global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs mlp, RenderWs w, const void* feat_,
+                                                           int f16) {
+  using namespace tc;
+  using S = Smem<NP>;
+  extern __shared__ __align__(1024) char sm[];
+  Bars& B = *(Bars*)(sm + S::bars);
+  uint32_t* err = &w.hdr[0];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the weights, split; biases and layer 3 in FP32
+  load_weights<NP>(sm + S::w1, kW1Bytes, mlp.w1, kHidden, mlp.in_dim, kK1);
+  load_weights<NP>(sm + S::w2, kW2Bytes, mlp.w2, kHidden, kHidden, kHidden);
+  float* b1s = (float*)(sm + S::b1);
+  float* l3 = (float*)(sm + S::l3);
+  float* b3s = (float*)(sm + S::b3);
+  for (int i = threadIdx.x; i < kHidden; i += kThreads) {
+    b1s[i] = mlp.b1[i];
+    float* p = l3 + 8 * (i >> 1) + (i & 1);
+    p[0] = mlp.b2[i];
+    p[2] = mlp.w3[i];
+    p[4] = mlp.w3[kHidden + i];
+    p[6] = mlp.w3[2 * kHidden + i];
+  }
+  if (threadIdx.x < 4) b3s[threadIdx.x] = threadIdx.x < 3 ? mlp.b3[threadIdx.x] : 0.0f;
+  if (threadIdx.x == 0) {
+    for (int b = 0; b < 2; b++) {
+      mbar_init(&B.xfull[b], kGatWarps);
+      mbar_init(&B.l1done[b], 1);
+      mbar_init(&B.l2done[b], 1);
+      mbar_init(&B.dfree[b], kEpiWarps);
+    }
+    for (int c = 0; c < kChunks; c++) {
+      mbar_init(&B.afull[c], kEpiWarps);
+      mbar_init(&B.cdone[c], 1);
+    }
+    for (int k = 0; k < kMeta; k++) {
+      mbar_init(&B.zfull[k], kEpiWarps / 2);
+      mbar_init(&B.mfull[k], kGatWarps);
+    }
+    mbar_init(&B.last, 1);
+    fence_mbar_init();
+  }
+  fence_proxy_async();
+  if (wid == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&B.tmem)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = B.tmem;
+  const uint32_t dcol = tmem + Tmem<NP>::acc;  // accumulator of tile i: dcol + 128 (i & 1)
+
+  const uint32_t n_tiles = w.hdr[1];
+  const uint32_t per = (n_tiles + gridDim.x - 1) / gridDim.x;
+  const uint32_t t0 = min(n_tiles, blockIdx.x * per), n = min(n_tiles, t0 + per) - t0;
+
+  if (wid < kE2) {
+    // ------------------------------------------------------------------ E1: layer 1 -> h1
+    regs_up<kRegsE1>();
+    const int h = wid >> 2;
+    const uint32_t lanes = (uint32_t)((wid & 3) * 32) << 16;
+    bool alive = true;
+    for (uint32_t i = 0; i < n && alive; i++) {
+      if (!(alive = warp_wait(&B.l1done[i & 1], (i >> 1) & 1, err))) break;
+      fence_after();
+      float v[64];
+      load_half(dcol + 128u * (i & 1) + lanes, h, v);  // all of it: layer 2 overwrites these columns
+#pragma unroll
+      for (int q4 = 0; q4 < 4; q4++) {  // 16 units at a time, 4 / kChunks of them per chunk
+        constexpr int kPer = 4 / kChunks;
+        const int c = q4 / kPer;
+        const float4* b4 = reinterpret_cast<const float4*>(b1s + 32 * q4 + 16 * h);
+        uint32_t o[NP][8];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          const float4 b = b4[q];
+          const float* z = v + 16 * q4 + 4 * q;
+          const float2 u0 = add2(make_float2(z[0], z[1]), make_float2(b.x, b.y));
+          const float2 u1 = add2(make_float2(z[2], z[3]), make_float2(b.z, b.w));
+          uint32_t p0[NP], p1[NP];
+          split2<NP>(make_float2(fmaxf(u0.x, 0.0f), fmaxf(u0.y, 0.0f)), p0);
+          split2<NP>(make_float2(fmaxf(u1.x, 0.0f), fmaxf(u1.y, 0.0f)), p1);
+#pragma unroll
+          for (int k = 0; k < NP; k++) {
+            o[k][2 * q] = p0[k];
+            o[k][2 * q + 1] = p1[k];
+          }
+        }
+        // the hi part's other buffer is free (layer 2 of tile i - 2 was issued before layer 1 of tile i)
+        tmem_st8(tmem + lanes + h1_col(0, i) + 16u * q4 + 8u * h, o[0]);
+        if (i > 0 && q4 % kPer == 0) {  // the smaller parts of tile i - 1's chunk have been read
+          if (!(alive = warp_wait(&B.cdone[c], (i - 1) & 1, err))) break;
+          fence_after();
+        }
+#pragma unroll
+        for (int k = 1; k < NP; k++) tmem_st8(tmem + lanes + h1_col(k, i) + 16u * q4 + 8u * h, o[k]);
+        if (q4 % kPer == kPer - 1) {
+          tmem_wait_st();
+          fence_before();
+          warp_arrive(&B.afull[c]);
+        }
+      }
+    }
+  } else if (wid < kG) {
+    // ------------------------------------------------------------------ E2: layer 2 -> layer 3 -> record
+    regs_up<kRegsE2>();
+    const int h = (wid - kE2) >> 2, m = (wid & 3) * 32 + lane;
+    const uint32_t lanes = (uint32_t)((wid & 3) * 32) << 16;
+    float4* zbuf = (float4*)(sm + S::z);
+    const float4* meta = (const float4*)(sm + S::meta);
+    for (uint32_t t = 0; t < n; t++) {
+      if (!warp_wait(&B.l2done[t & 1], (t >> 1) & 1, err)) break;
+      if (!warp_wait(&B.mfull[t % kMeta], (t / kMeta) & 1, err)) break;
+      fence_after();
+      const float4 md = meta[(t % kMeta) * kTile + m];
+      float v[64];
+      load_half(dcol + 128u * (t & 1) + lanes, h, v);  // all of it, to free the accumulator at once
+      fence_before();
+      warp_arrive(&B.dfree[t & 1]);
+      float2 z0 = make_float2(0.f, 0.f), z1 = z0, z2 = z0;
+      const float4* l4 = reinterpret_cast<const float4*>(l3) + 16 * h;  // two per pair of units
+#pragma unroll
+      for (int q = 0; q < 32; q++) {
+        const float4 a = l4[32 * (q / 8) + 2 * (q % 8)], b = l4[32 * (q / 8) + 2 * (q % 8) + 1];
+        float2 u = add2(make_float2(v[2 * q], v[2 * q + 1]), make_float2(a.x, a.y));
+        u.x = fmaxf(u.x, 0.0f);
+        u.y = fmaxf(u.y, 0.0f);
+        z0 = fma2(make_float2(a.z, a.w), u, z0);
+        z1 = fma2(make_float2(b.x, b.y), u, z1);
+        z2 = fma2(make_float2(b.z, b.w), u, z2);
+      }
+      float4* zp = &zbuf[(t % kMeta) * kTile + m];
+      if (h) {
+        *zp = make_float4(z0.x + z0.y, z1.x + z1.y, z2.x + z2.y, 0.0f);
+        warp_arrive(&B.zfull[t % kMeta]);
+      } else {
+        if (!warp_wait(&B.zfull[t % kMeta], (t / kMeta) & 1, err)) break;
+        const float4 o = *zp;
+        const uint32_t rid = __float_as_uint(md.x);
+        if (rid != 0xffffffffu)
+          w.rec_c[rid] = make_float4(sigmoid_f(z0.x + z0.y + o.x + b3s[0]), sigmoid_f(z1.x + z1.y + o.y + b3s[1]),
+                                     sigmoid_f(z2.x + z2.y + o.z + b3s[2]), md.y);
+      }
+    }
+  } else if (wid < kM) {
+    // ------------------------------------------------------------------ G: the input rows
+    const int m = (wid & 3) * 32 + lane;
+    const uint32_t grp = (uint32_t)(wid - kG) / kGatWarps;  // takes tiles grp, grp + 2, ...
+    const int C = CC ? CC : g.C, n_freq = NF ? NF : mlp.n_freq, Br = g.brick;
+    float4* meta = (float4*)(sm + S::meta);
+    uint4 td = make_uint4(0u, 0u, 0u, 0u);
+    float4 pw = make_float4(0.f, 0.f, 0.f, 0.f), qd = pw;
+    auto fetch = [&](uint32_t i) {
+      td = w.tile[t0 + i];
+      if (m < (int)(td.y & 0xFFu)) {
+        pw = w.srt[td.x + m].pw;
+        qd = w.srt[td.x + m].qd;
+      }
+    };
+    if (grp < n) fetch(grp);
+    for (uint32_t i = grp; i < n; i += 2) {
+      const bool valid = m < (int)(td.y & 0xFFu);
+      float x[kK1];
+#pragma unroll
+      for (int k = 0; k < kK1; k++) x[k] = 0.0f;
+      float d[3] = {0.f, 0.f, 0.f};
+      float4 md = make_float4(__uint_as_float(0xffffffffu), 0.f, 0.f, 0.f);
+      if (valid) {
+        const float p[3] = {pw.x, pw.y, pw.z};
+        d[0] = qd.y;
+        d[1] = qd.z;
+        d[2] = qd.w;
+        md.x = qd.x;
+        md.y = pw.w;
+        const int bx = (int)(td.w & 0xFFFFu), by = (int)(td.w >> 16), bz = (int)((td.y >> 8) & 0x1FFFu);
+        int i0[3];
+        float f[3];
+        const bool in = index_sample(g, p, i0, f);
+        const int l[3] = {i0[0] - bx * Br, i0[1] - by * Br, i0[2] - bz * Br};
+        if (!(in && l[0] >= 0 && l[0] < Br && l[1] >= 0 && l[1] < Br && l[2] >= 0 && l[2] < Br))
+          set_err(err, kErrInternal);
+        else if (f16)
+          gather<__half, CC>(g, (const __half*)feat_, i0, f, x);
+        else
+          gather<float, CC>(g, (const float*)feat_, i0, f, x);
+      }
+      if (i + 2 < n) fetch(i + 2);
+      if (CC && NF && valid) encode<NF>(d, x + CC);
+      // x's buffer: layer 1 of tile i - 2 has read it
+      if (i >= 2 && !warp_wait(&B.l1done[i & 1], ((i >> 1) - 1) & 1, err)) break;
+      char* xb = sm + S::x + (int)(i & 1) * NP * kXBytes;
+#pragma unroll
+      for (int k0 = 0; k0 < kK1; k0 += 8) {
+        uint4 q[NP];
+        split_row<NP>(x + k0, q);
+#pragma unroll
+        for (int p = 0; p < NP; p++) *reinterpret_cast<uint4*>(xb + p * kXBytes + kmaj_off(m, k0, kK1)) = q[p];
+      }
+      if (!(CC && NF) && valid) {
+        // channels known at run time only: the encoding is written over columns C .. element by element
+        constexpr int F = (kK1 - 4) / 6;  // most frequencies with one channel
+        float e[3 + 6 * F + 1];
+        e[3 + 6 * F] = 0.0f;
+        encode<F>(d, e);
+        const int ne = 3 + 6 * n_freq;
+#pragma unroll
+        for (int j = 0; j < 3 + 6 * F; j += 2) {
+          uint32_t p[NP];
+          split2<NP>(make_float2(e[j], e[j + 1]), p);
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            const int k = C + j + u;
+            if (j + u < ne)
+#pragma unroll
+              for (int a = 0; a < NP; a++)
+                *reinterpret_cast<uint16_t*>(xb + a * kXBytes + kmaj_off(m, 0, kK1) + (k >> 3) * 128 + (k & 7) * 2) =
+                    (uint16_t)(p[a] >> (16 * u));
+          }
+        }
+      }
+      meta[(i % kMeta) * kTile + m] = md;
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) {
+        arrive(&B.xfull[i & 1]);
+        arrive(&B.mfull[i % kMeta]);
+      }
+    }
+  } else {
+    // ------------------------------------------------------------------ M: the MMAs
+    regs_down<kRegsM>();
+    if (wid == kM && n) issue_mmas<NP>(sm, B, tmem, n, err);
+  }
+  fence_before();
+  __syncthreads();
+  if (wid == 0) {
+    fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+  }
+}
+template <int NP, int CC, int NF>
+static cicero_status launch(const cicero_grid* grid, const GridGeo& geo, const MlpPtrs& mlp, const RenderWs& ws,
+                            cudaStream_t st) {
+  auto kern = k_mlp_split<NP, CC, NF>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<NP>::bytes);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_mlp_split)");
+  {
+    ProfScope ps(kStGatherMlp, st);
+    kern<<<num_sms(), kThreads, Smem<NP>::bytes, st>>>(geo, mlp, ws, grid->features, grid->dtype == CICERO_F16);
+  }
+  count_launches(1);
+  e = cudaGetLastError();
+  return e == cudaSuccess ? CICERO_OK : cuda_fail(e, "k_mlp_split");
+}
+
+}  // namespace ms
+
+cicero_status launch_mlp_split(const cicero_grid* grid, const GridGeo& geo, int parts, const MlpPtrs& mlp,
+                               const RenderWs& ws, cudaStream_t st) {
+  const bool c12 = geo.C == 12 && mlp.n_freq == 4;
+  if (parts == 3)
+    return c12 ? ms::launch<3, 12, 4>(grid, geo, mlp, ws, st) : ms::launch<3, 0, 0>(grid, geo, mlp, ws, st);
+  return c12 ? ms::launch<2, 12, 4>(grid, geo, mlp, ws, st) : ms::launch<2, 0, 0>(grid, geo, mlp, ws, st);
+}
+
+}  // namespace cicero

@@ -9,9 +9,9 @@
 //                     per thread), tile offsets per brick and the tile list
 //   K3 k_scatter      counting sort of the records by key, moving their payload into (brick,
 //                     octant) order as 32-byte records: the Ray Index Table
-//   K5 k_gather_mlp_f32 / mlp_tc.cu
-//                     per brick: one TMA copy of the brick (+1 vertex halo) into shared memory,
-//                     trilinear feature gathering from there, view encoding and the MLP
+//   K5 mlp_tc.cu      per brick: one TMA copy of the brick (+1 vertex halo) into shared memory,
+//                     trilinear feature gathering from there, view encoding and the BF16 MLP
+//      mlp_split.cu   the FP32-class MLPs: features from global memory, operands split into BF16 parts
 //   K6 k_composite    per ray, in slot order: rgb = sum w c + T_end bg
 #include <cuda_runtime.h>
 
@@ -851,63 +851,7 @@ __global__ void __launch_bounds__(256, 4) k_scatter(RaySrc src, RenderWs w) {
 }
 
 // -------------------------------------------------------------------------------------------
-// K5 (FP32): Feature Gathering from the staged brick and an FP32 SIMT MLP over 128-sample tiles.
-
-template <typename T>
-__device__ __forceinline__ void tri_smem(const T* tile, int vb, int vx, int C, const int l[3], const float f[3],
-                                         float* out) {
-  const float fx = f[0], fy = f[1], fz = f[2];
-  float wc[8];
-  wc[0] = (1.f - fx) * (1.f - fy) * (1.f - fz);
-  wc[1] = fx * (1.f - fy) * (1.f - fz);
-  wc[2] = (1.f - fx) * fy * (1.f - fz);
-  wc[3] = fx * fy * (1.f - fz);
-  wc[4] = (1.f - fx) * (1.f - fy) * fz;
-  wc[5] = fx * (1.f - fy) * fz;
-  wc[6] = (1.f - fx) * fy * fz;
-  wc[7] = fx * fy * fz;
-  for (int c = 0; c < C; c++) out[c] = 0.0f;
-#pragma unroll
-  for (int q = 0; q < 8; q++) {
-    const int x = l[0] + (q & 1), y = l[1] + ((q >> 1) & 1), z = l[2] + (q >> 2);
-    const T* v = tile + ((size_t)(z * vb + y) * vx + x) * C;
-    if constexpr (sizeof(T) == 4) {
-      if (C == 12) {
-        const float4* v4 = reinterpret_cast<const float4*>(v);
-#pragma unroll
-        for (int u = 0; u < 3; u++) {
-          float4 a = v4[u];
-          out[4 * u + 0] += wc[q] * a.x;
-          out[4 * u + 1] += wc[q] * a.y;
-          out[4 * u + 2] += wc[q] * a.z;
-          out[4 * u + 3] += wc[q] * a.w;
-        }
-        continue;
-      }
-    } else {
-      if (C == 12) {
-        const uint2* v2 = reinterpret_cast<const uint2*>(v);
-#pragma unroll
-        for (int u = 0; u < 3; u++) {
-          uint2 a = v2[u];
-          float2 lo = __half22float2(*reinterpret_cast<__half2*>(&a.x));
-          float2 hi = __half22float2(*reinterpret_cast<__half2*>(&a.y));
-          out[4 * u + 0] += wc[q] * lo.x;
-          out[4 * u + 1] += wc[q] * lo.y;
-          out[4 * u + 2] += wc[q] * hi.x;
-          out[4 * u + 3] += wc[q] * hi.y;
-        }
-        continue;
-      }
-    }
-    for (int c = 0; c < C; c++) {
-      float vv;
-      if constexpr (sizeof(T) == 4) vv = v[c];
-      else vv = __half2float(v[c]);
-      out[c] += wc[q] * vv;
-    }
-  }
-}
+// FP32 SIMT MLP over 128-sample tiles: the backward's fix-up of uncertain samples and cicero_mlp_eval.
 
 constexpr int kK1 = kMaxIn;  // padded input width of layer 1
 
@@ -919,14 +863,10 @@ struct F32Smem {
   static constexpr int b1 = w3 + 3 * kHidden * 4;                // [128]
   static constexpr int b2 = b1 + kHidden * 4;                    // [128]
   static constexpr int b3 = b2 + kHidden * 4;                    // [4]
-  static constexpr int x = b3 + 16;                              // [48][128] inputs, buffer 0
+  static constexpr int x = b3 + 16;                              // [48][128] inputs
   static constexpr int h = x + kK1 * kTile * 4;                  // [128][128]
-  static constexpr int bar = ((h + kHidden * kTile * 4 + 127) / 128) * 128;  // mbarrier (8 B, pad 128)
-  static constexpr int x2 = bar + 128;                           // [48][128] inputs, buffer 1
-  // brick tile (TMA destination, 128-B aligned): after buffer 1, or in its place with one buffer
-  static constexpr int tile = x2 + kK1 * kTile * 4;
-  static constexpr int tile1 = x2;
-  static_assert(tile % 128 == 0 && tile1 % 128 == 0, "TMA destination must be 128-byte aligned");
+  static constexpr int end = ((h + kHidden * kTile * 4 + 127) / 128) * 128;
+  static constexpr int masks = end;                              // the fix-up's ReLU bytes [2][16][128]
 };
 
 // acc[i][j]: rows {tm*4+i, 64+tm*4+(i-4)}, cols {tn*4+j, 64+tn*4+(j-4)}; A, B k-major [K][128].
@@ -1002,33 +942,14 @@ __device__ void load_mlp_f32_smem(char* sm, const MlpPtrs& m) {
   if (threadIdx.x < 4) b3[threadIdx.x] = threadIdx.x < 3 ? m.b3[threadIdx.x] : 0.0f;
 }
 
-// Named barriers of the FP32 kernels: the 256 MLP threads among themselves, and the hand-off of
-// the two input buffers between the producer warps and the MLP threads (full: the producers
-// arrive, the MLP threads wait; empty: the reverse).
-constexpr int kBarMlp = 1, kBarProd = 2, kBarFull0 = 3, kBarEmpty0 = 5;
-constexpr int kMlpThreads = 256, kProdThreads = 128;
+// Named barrier of the FP32 kernels' 256 MLP threads.
+constexpr int kBarMlp = 1;
+constexpr int kMlpThreads = 256;
 __device__ __forceinline__ void nbar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ bool nbar_sync_and(int id, int n, bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 p, %1, 0;\n\t"
-      "bar.red.and.pred q, %2, %3, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)v), "r"(id), "r"(n)
-      : "memory");
-  return r != 0;
-}
-__device__ __forceinline__ void nbar_arrive(int id, int n) {
-  __threadfence_block();  // this thread's shared-memory accesses before the arrival
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
 
 // Three-layer MLP of the 128 samples whose inputs are in X [48][128] (rows in_dim.. zero);
 // threads < 128 return c of sample m = threadIdx.x.  Run by the 256 MLP threads (threadIdx.x < 256), which synchronise on
-// their own named barrier; with empty_id > 0 they also arrive on that barrier (with the producers,
-// kMlpThreads + kProdThreads) once layer 1 has read X.
+// their own named barrier.
 // This thread's ReLU bits of one layer into msk [16][128] bytes: byte (tn, m) holds units
 // tn * 4 + j (bit j) and 64 + tn * 4 + j (bit 4 + j) of sample m, as relu(acc + bias) > 0 decides.
 __device__ __forceinline__ void store_relu_bits(const float acc[8][8], const float* bias, uint8_t* msk, int tm,
@@ -1043,7 +964,7 @@ __device__ __forceinline__ void store_relu_bits(const float acc[8][8], const flo
 }
 
 // msk (may be NULL): [2][16][128] bytes receiving the ReLU masks of layers 1 and 2 (store_relu_bits).
-__device__ __forceinline__ void mlp_f32_tile(char* sm, const float* X, float c[3], int in_dim, int empty_id = 0,
+__device__ __forceinline__ void mlp_f32_tile(char* sm, const float* X, float c[3], int in_dim,
                                              uint8_t* msk = nullptr) {
   const float* w1t = (const float*)(sm + F32Smem::w1t);
   const float* w2t = (const float*)(sm + F32Smem::w2t);
@@ -1062,7 +983,6 @@ __device__ __forceinline__ void mlp_f32_tile(char* sm, const float* X, float c[3
   if (msk) store_relu_bits(acc, b1, msk, tm, tn);
   simt_epilogue(acc, b1, H, tm, tn);
   nbar_sync(kBarMlp, kMlpThreads);
-  if (empty_id) nbar_arrive(empty_id, kMlpThreads + kProdThreads);  // X may be refilled
 #pragma unroll
   for (int i = 0; i < 8; i++)
 #pragma unroll
@@ -1111,124 +1031,9 @@ __device__ __forceinline__ void mlp_f32_tile(char* sm, const float* X, float c[3
   }
 }
 
-// K5f: FP32 Feature Gathering + Computation.  Warps 0-7 run the MLP of tile t while warps 8-11
-// (producers, one thread per sample row) gather tile t + 1 into the other input buffer: staged
-// brick (TMA, reloaded when the brick changes) -> trilinear features + direction encoding.  With
-// nbuf = 1 (a brick too large for two buffers) the producers wait until layer 1 of tile t has read
-// the single buffer.  The buffers are handed over with named barriers (full / empty, alternating
-// between two ids per tile so that consecutive generations never mix); a producer that runs into
-// a timeout keeps taking part in them (with zero inputs), so the MLP threads never wait on a
-// barrier that cannot complete.
-template <typename T>
-__global__ void __launch_bounds__(kMlpThreads + kProdThreads, 1)
-    k_gather_mlp_f32(GridGeo g, int S, MlpPtrs mlp, RenderWs w, const __grid_constant__ CUtensorMap fmap, int vb,
-                     int vx, int box_bytes, int nbuf) {
-  extern __shared__ __align__(128) char sm[];
-  uint64_t* bar = (uint64_t*)(sm + F32Smem::bar);
-  T* tile = (T*)(sm + (nbuf == 2 ? F32Smem::tile : F32Smem::tile1));
-  // the ReLU masks of two tiles, after the brick tile (present only when the launch records masks)
-  uint8_t* mask_smem = (uint8_t*)tile + ((box_bytes + 127) & ~127);
-  load_mlp_f32_smem(sm, mlp);
-  if (threadIdx.x == 0) {
-    mbar_init(bar, 1);
-    fence_mbar_init();
-  }
-  __syncthreads();
-  const uint32_t n_tiles = w.hdr[1];
-  const uint32_t per = (n_tiles + gridDim.x - 1) / gridDim.x;
-  const uint32_t t_begin = blockIdx.x * per, t_end = min(n_tiles, t_begin + per);
-  const uint32_t n = t_end > t_begin ? t_end - t_begin : 0;
-  if (threadIdx.x >= kMlpThreads) {
-    // ------------------------------------------------------------------ producers
-    const int m = threadIdx.x - kMlpThreads;
-    const int B = g.brick, C = g.C;
-    int loaded = -1;
-    uint32_t phase = 0;
-    bool alive = true;
-    for (uint32_t i = 0; i < n; i++) {
-      const int b = i & 1;
-      float* X = (float*)(sm + ((i % nbuf) ? F32Smem::x2 : F32Smem::x));
-      // layer 1 of tile i - nbuf, the buffer's last user, is done with it
-      if (i >= (uint32_t)nbuf) nbar_sync(kBarEmpty0 + ((i - nbuf) & 1), kMlpThreads + kProdThreads);
-      const uint4 td = w.tile[t_begin + i];
-      const uint32_t start = td.x;
-      const int mcnt = (int)(td.y & 0xFFu);
-      const int bx = (int)(td.w & 0xFFFFu), by = (int)(td.w >> 16), bz = (int)((td.y >> 8) & 0x1FFFu);
-      if (alive && (int)td.z != loaded) {
-        nbar_sync(kBarProd, kProdThreads);  // every producer is done with the staged brick
-        if (m == 0) {
-          mbar_expect_tx(bar, (uint32_t)box_bytes);
-          tma_load_3d(tile, &fmap, bx * B * C, by * B, bz * B, bar);
-        }
-        alive = nbar_sync_and(kBarProd, kProdThreads, mbar_wait(bar, phase, &w.hdr[0]));
-        if (alive) phase ^= 1u;
-        loaded = (int)td.z;
-      }
-      if (alive && m < mcnt) {
-        const float4 pw = w.srt[start + m].pw;
-        const float4 dd = w.srt[start + m].qd;
-        const float p[3] = {pw.x, pw.y, pw.z}, d[3] = {dd.y, dd.z, dd.w};
-        float f[3], feat[24], e[3 + 6 * 7];
-        int i0[3];
-        const bool ok = index_sample(g, p, i0, f);
-        const int l[3] = {i0[0] - bx * B, i0[1] - by * B, i0[2] - bz * B};
-        if (!ok || l[0] < 0 || l[0] >= B || l[1] < 0 || l[1] >= B || l[2] < 0 || l[2] >= B) {
-          set_err(&w.hdr[0], kErrInternal);
-          for (int c = 0; c < C; c++) X[c * kTile + m] = 0.0f;
-        } else {
-          tri_smem<T>(tile, vb, vx, C, l, f, feat);
-          for (int c = 0; c < C; c++) X[c * kTile + m] = feat[c];
-        }
-        encode_dir(d, mlp.n_freq, e);
-        const int ne = 3 + 6 * mlp.n_freq;
-        for (int j = 0; j < ne; j++) X[(C + j) * kTile + m] = e[j];
-        for (int j = C + ne; j < kK1; j++) X[j * kTile + m] = 0.0f;
-      } else {
-        for (int j = 0; j < kK1; j++) X[j * kTile + m] = 0.0f;
-      }
-      nbar_arrive(kBarFull0 + b, kMlpThreads + kProdThreads);
-    }
-    // the MLP threads' last releases of each buffer, so that every barrier is left balanced
-    for (uint32_t i = n >= (uint32_t)nbuf ? n - nbuf : 0; i < n; i++)
-      nbar_sync(kBarEmpty0 + (i & 1), kMlpThreads + kProdThreads);
-    return;
-  }
-  // -------------------------------------------------------------------- MLP threads
-  for (uint32_t i = 0; i < n; i++) {
-    const int b = i & 1;
-    const float* X = (const float*)(sm + ((i % nbuf) ? F32Smem::x2 : F32Smem::x));
-    const uint4 td = w.tile[t_begin + i];
-    const uint32_t start = td.x;
-    const int mcnt = (int)(td.y & 0xFFu);
-    nbar_sync(kBarFull0 + b, kMlpThreads + kProdThreads);  // the producers have filled X
-    float c[3];
-    // with a backward to follow, the layers' ReLU masks too (two buffers by tile parity: a thread
-    // cannot write tile i + 2's masks before every thread has passed tile i + 1's first barrier,
-    // which follows its reads of tile i's)
-    uint8_t* msk = w.rec_mask ? mask_smem + (i & 1) * 32 * kTile : nullptr;
-    mlp_f32_tile(sm, X, c, mlp.in_dim, kBarEmpty0 + b, msk);
-    const int m = threadIdx.x;
-    if (m < kTile && m < mcnt) {
-      const uint32_t rid = __float_as_uint(w.srt[start + m].qd.x);
-      w.rec_c[rid] = make_float4(c[0], c[1], c[2], w.srt[start + m].pw.w);
-      if (msk) {
-        uint32_t v[8];
-#pragma unroll
-        for (int q = 0; q < 8; q++) {  // word q: bytes tn = 4 q' .. of layer q / 4
-          const uint8_t* src = msk + (q >> 2) * 16 * kTile + (q & 3) * 4 * kTile + m;
-          v[q] = (uint32_t)src[0] | ((uint32_t)src[kTile] << 8) | ((uint32_t)src[2 * kTile] << 16) |
-                 ((uint32_t)src[3 * kTile] << 24);
-        }
-        w.rec_mask[2 * (size_t)rid] = make_uint4(v[0], v[1], v[2], v[3]);
-        w.rec_mask[2 * (size_t)rid + 1] = make_uint4(v[4], v[5], v[6], v[7]);
-      }
-    }
-  }
-}
-
 // The samples that the backward's tensor-core forward recompute (k_fwd_x3) listed (a ReLU
 // pre-activation within its error estimate of zero for the split-BF16 products), recomputed with the FP32
-// MLP of K5f: (c, w) and both ReLU masks overwritten.  The list holds sorted record indices
+// MLP (mlp_f32_tile): (c, w) and both ReLU masks overwritten.  The list holds sorted record indices
 // (rec_key, count in hdr[4]); 128 samples per step, features interpolated from global memory.
 // Launched only after k_fwd_x3, so C <= 16.
 template <typename T>
@@ -1236,7 +1041,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_fwd_fix(GridGeo g, MlpPtrs m
                                                            const T* __restrict__ feat) {
   extern __shared__ __align__(128) char sm[];
   float* X = (float*)(sm + F32Smem::x);
-  uint8_t* msk = (uint8_t*)(sm + F32Smem::x2);  // [2][16][128] ReLU bytes (store_relu_bits)
+  uint8_t* msk = (uint8_t*)(sm + F32Smem::masks);  // [2][16][128] ReLU bytes (store_relu_bits)
   load_mlp_f32_smem(sm, mlp);
   const uint32_t n = w.hdr[4];
   const int C = g.C, m = threadIdx.x;
@@ -1289,7 +1094,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_fwd_fix(GridGeo g, MlpPtrs m
     }
     __syncthreads();
     float c[3];
-    mlp_f32_tile(sm, X, c, mlp.in_dim, 0, msk);
+    mlp_f32_tile(sm, X, c, mlp.in_dim, msk);
     if (valid) {
       const uint32_t rid = __float_as_uint(w.srt[si].qd.x);
       w.rec_c[rid] = make_float4(c[0], c[1], c[2], w.srt[si].pw.w);
@@ -1309,7 +1114,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_fwd_fix(GridGeo g, MlpPtrs m
 template <typename T>
 static cicero_status launch_fwd_fix(const GridGeo& geo, const MlpPtrs& mlp, const RenderWs& ws, const void* feat,
                                     cudaStream_t st) {
-  const int smem = F32Smem::x2 + 2 * 16 * kTile;
+  const int smem = F32Smem::masks + 2 * 16 * kTile;
   cudaError_t e = cudaFuncSetAttribute(k_fwd_fix<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_fwd_fix)");
   {
@@ -1542,26 +1347,9 @@ static int blocks_for_warps(long long warps, int per_sm) {
   return (int)blocks;
 }
 
-template <typename T>
-static cicero_status launch_f32(const GridGeo& geo, int S, const MlpPtrs& mlp, const RenderWs& ws,
-                                const CUtensorMap& map, const BrickBox& box, cudaStream_t st) {
-  const int masks = ws.rec_mask ? 2 * 32 * kTile : 0;  // ReLU masks of two tiles for the backward
-  const int boxa = (box.box_bytes + 127) & ~127;
-  const int nbuf = F32Smem::tile + boxa + masks <= 227 * 1024 ? 2 : 1;  // two input buffers when they fit
-  const int smem = (nbuf == 2 ? F32Smem::tile : F32Smem::tile1) + boxa + masks;
-  if (smem > 227 * 1024) return fail(CICERO_ERR_UNSUPPORTED, "brick too large for the FP32 feature-computation kernel");
-  auto kern = k_gather_mlp_f32<T>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_gather_mlp_f32)");
-  {
-    ProfScope ps(kStGatherMlp, st);
-    kern<<<num_sms(), kMlpThreads + kProdThreads, smem, st>>>(geo, S, mlp, ws, map, box.vb, box.vx, box.box_bytes,
-                                                                   nbuf);
-  }
-  count_launches(1);
-  e = cudaGetLastError();
-  return e == cudaSuccess ? CICERO_OK : cuda_fail(e, "k_gather_mlp_f32");
-}
+// The brick sizes an FP32 render takes: those whose box fits in shared memory beside the 183,040 bytes
+// that an FP32 MLP's weights and buffers take.  k_mlp_split stages no brick; the limit is the interface's.
+static bool f32_brick_fits(const BrickBox& box) { return 183040 + ((box.box_bytes + 127) & ~127) <= 227 * 1024; }
 
 cicero_status run_render(const cicero_grid* grid, const MlpPtrs& mlp, const RenderPlan& plan, const RaySrc& src,
                          const RenderWs& ws, const OutBufs& out, bool stop_after_bucketing, cudaStream_t st,
@@ -1607,7 +1395,7 @@ cicero_status run_render(const cicero_grid* grid, const MlpPtrs& mlp, const Rend
     // split-BF16 tensor-core MLP, features read from global memory (no staged brick)
     if (!fwd_x3_supported(geo, mlp))
       return fail(CICERO_ERR_UNSUPPORTED, "the split-BF16 MLP takes at most 16 feature channels");
-    s = launch_fwd_x3(grid, geo, mlp, ws, st);  // colours only (no masks: rec_mask is NULL)
+    s = launch_mlp_split(grid, geo, 2, mlp, ws, st);
   } else if (ws.rec_mask && fwd_x3_supported(geo, mlp)) {
     // a backward follows: colours and ReLU masks only, on the tensor cores, then the uncertain
     // samples again in FP32
@@ -1620,8 +1408,8 @@ cicero_status run_render(const cicero_grid* grid, const MlpPtrs& mlp, const Rend
   } else if (plan.precision == CICERO_MLP_BF16) {
     s = launch_gather_mlp_bf16(grid, geo, plan.mlp_groups, mlp, ws, map, box, st);
   } else {
-    s = f16 ? launch_f32<__half>(geo, plan.S, mlp, ws, map, box, st)
-            : launch_f32<float>(geo, plan.S, mlp, ws, map, box, st);
+    s = f32_brick_fits(box) ? launch_mlp_split(grid, geo, 3, mlp, ws, st)
+                            : fail(CICERO_ERR_UNSUPPORTED, "brick too large for the FP32 feature-computation kernel");
   }
   if (s != CICERO_OK) return s;
   if (!out.rgb[0]) return CICERO_OK;  // the backward only needs the per-sample records
@@ -1711,7 +1499,7 @@ __global__ void __launch_bounds__(256, 1) k_mlp_eval_f32(MlpPtrs mlp, const floa
 }
 
 cicero_status launch_mlp_eval_f32(const MlpPtrs& mlp, const float* x, int M, float* c, cudaStream_t st) {
-  const int smem = F32Smem::bar;
+  const int smem = F32Smem::end;
   cudaError_t e = cudaFuncSetAttribute(k_mlp_eval_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_mlp_eval_f32)");
   const int ntile = (M + kTile - 1) / kTile;

@@ -1,6 +1,7 @@
-"""Feature-channel layouts of the BF16 gather + MLP kernels against the FP64 oracle (2e-2, the path's
+"""Feature-channel layouts of the gather + MLP kernels against the FP64 oracle.  BF16 (2e-2, the path's
 tolerance): every specialised channel count and the general kernel, with the features from staged bricks
-and, where those leave room for fewer tiles in flight, from global memory."""
+and, where those leave room for fewer tiles in flight, from global memory.  FP32 and split BF16: the
+pipelined tensor-core kernel, from a single tile to several per SM."""
 import numpy as np
 import pytest
 
@@ -57,3 +58,36 @@ def test_batch_channel_layouts(cc, C, brick):
         one = gpu_render(cc, None, None, cam, cam.sampling, cc.MLP_BF16, brick, dev_grid=g, dev_mlp=m)
         assert (rgb.cpu().numpy().astype(np.float64) == one["rgb"]).all()
         assert (depth.cpu().numpy().astype(np.float64) == one["depth"]).all()
+
+
+# |d rgb| <= sum of weights (<= 1) x sigmoid' (1/4) x |d z3|.  FP32: six products of three BF16 parts leave
+# ~2^-24 of each term, and the accumulations ~11 x 2^-24 of a sum of a few units: ~1e-6, beside the march's
+# ~3e-7; split BF16 leaves ~2^-17 of each term: ~1.5e-5.
+TOL_SPLIT = {0: 5e-6, 2: 2e-5}
+
+
+@pytest.mark.parametrize("precision,C,n_freq,dtype", [
+    (0, 12, 4, np.float16), (0, 12, 4, np.float32), (0, 8, 4, np.float16), (0, 21, 4, np.float32), (0, 1, 7, np.float32),
+    (0, 5, 0, np.float32), (0, 13, 2, np.float32), (2, 12, 4, np.float16), (2, 16, 4, np.float32), (2, 3, 7, np.float32),
+    (2, 6, 4, np.float16)])
+def test_split_channel_layouts(cc, orc, precision, C, n_freq, dtype):
+    g = scenes.make_grid(32, C, 4, seed=600 + C, dtype=dtype)
+    m = scenes.make_mlp(C, seed=700 + C, n_freq=n_freq, random_bias=True)
+    cam = scenes.orbit_camera(29, 33, az_deg=70.0, sampling=scenes.sampling_uniform(48))
+    ref = orc.render(g, m, cam.sampling, cam=cam)
+    check_render(gpu_render(cc, g, m, cam, cam.sampling, precision, 4), ref, TOL_SPLIT[precision])
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+@pytest.mark.parametrize("side,n_samples", [(1, 1), (2, 40), (12, 16), (40, 40), (120, 64)])
+def test_split_tile_counts(cc, orc, precision, side, n_samples):
+    """Tiles per SM from none or one to several, bricks of 16 (full tiles) and 4 (ragged ones)."""
+    g, m = scenes.make_grid(48, 12, 6, seed=81), scenes.make_mlp(12, seed=82, random_bias=True)
+    cam = scenes.orbit_camera(side, side, az_deg=20.0, sampling=scenes.sampling_uniform(n_samples))
+    pix = (scenes.splitmix64(83, 200) % np.uint64(side * side)).astype(np.int32) if side > 40 else None
+    ref = orc.render(g, m, cam.sampling, cam=cam, pix=pix)
+    for brick in (4, 8):
+        out = gpu_render(cc, g, m, cam, cam.sampling, precision, brick)
+        if pix is not None:
+            out = {k: v[pix] for k, v in out.items()}
+        check_render(out, ref, TOL_SPLIT[precision])
