@@ -125,35 +125,42 @@ struct Group {
   uint32_t ph_tma, ph_mma;
 };
 
-// Issue one layer (elected thread) and wait for it (whole group).  False on timeout.
-// Layers 0 and 1 read A from shared memory and accumulate into the group's columns [0, 128);
-// layer 2 reads A from the group's TMEM columns [0, 64) and accumulates into [64, 80).
-__device__ __forceinline__ bool run_layer(char* sm, Group& G, int layer, uint32_t* err) {
-  gsync(G.g);
-  if (G.m == 0) {
+// Issue one layer's MMAs and commit them to the group's mbarrier (the group's first warp, all lanes;
+// one elected lane issues).  Layers 0 and 1 read A from shared memory and accumulate into the group's
+// columns [0, 128); layer 2 reads A from the group's TMEM columns [0, 64) and accumulates into [64, 80).
+// A always has the K = 144 row-group stride (layer 0's A fills its first 48 columns); a K step of 16 is
+// 256 bytes.  The operands are made warp-uniform first: the instruction reads uniform registers, and
+// moving every descriptor there from a thread's own took ~10 instructions per MMA on every group's
+// critical path.
+template <int LAYER>
+__device__ __forceinline__ void issue_layer(char* sm, const Group& G) {
+  const uint32_t tmem = __shfl_sync(0xffffffffu, G.tmem, 0);
+  const uint32_t act = __shfl_sync(0xffffffffu, desc_lo(smem_u32(G.act), 128u), 0);
+  const uint32_t bar = __shfl_sync(0xffffffffu, smem_u32(G.bar_mma), 0);
+  if (elect_one()) {
     fence_after();
-    if (layer < 2) {
-      // descriptors built once; the next K step of 16 is 256 bytes on, +16 in the address field.
-      // A always has the K = 144 row-group stride (layer 1's A fills its first 48 columns).
-      const uint64_t da = smem_desc(smem_u32(G.act), 128u, kK2 * 16);
-      const uint64_t db = smem_desc(smem_u32(sm + (layer == 0 ? Smem::w1 : Smem::w2)), 128u,
-                                    (uint32_t)(layer == 0 ? kK1 : kK2) * 16);
-      const uint32_t idesc = idesc_bf16(kHidden);
-      if (layer == 0) {
+    if constexpr (LAYER < 2) {
+      constexpr uint32_t ahi = desc_hi(kK2 * 16), bhi = desc_hi((LAYER == 0 ? kK1 : kK2) * 16);
+      const uint32_t b = desc_lo(smem_u32(sm + (LAYER == 0 ? Smem::w1 : Smem::w2)), 128u);
 #pragma unroll
-        for (int s = 0; s < kK1 / 16; s++) mma_bf16(G.tmem, da + 16u * s, db + 16u * s, idesc, s > 0 ? 1u : 0u);
-      } else {
-#pragma unroll
-        for (int s = 0; s < kK2 / 16; s++) mma_bf16(G.tmem, da + 16u * s, db + 16u * s, idesc, s > 0 ? 1u : 0u);
-      }
+      for (int s = 0; s < (LAYER == 0 ? kK1 : kK2) / 16; s++)
+        mma_u<ahi, bhi, idesc_bf16(kHidden)>(tmem, act + 16u * s, b + 16u * s, s > 0 ? 1u : 0u);
     } else {
-      const uint64_t db = smem_desc(smem_u32(sm + Smem::w3), 128u, kHidden * 16);
+      const uint32_t b = desc_lo(smem_u32(sm + Smem::w3), 128u);
 #pragma unroll
       for (int s = 0; s < kHidden / 16; s++)
-        mma_bf16_ta(G.tmem + kL3Col, G.tmem + 8u * s, db + 16u * s, idesc_bf16(kN3), s > 0 ? 1u : 0u);
+        mma_u_ta<desc_hi(kHidden * 16), idesc_bf16(kN3)>(tmem + kL3Col, tmem + 8u * s, b + 16u * s, s > 0 ? 1u : 0u);
     }
-    mma_commit(G.bar_mma);
+    mma_commit_at(bar);
   }
+  __syncwarp();
+}
+
+// Issue one layer and wait for it (whole group).  False on timeout.
+template <int LAYER>
+__device__ __forceinline__ bool run_layer(char* sm, Group& G, uint32_t* err) {
+  gsync(G.g);
+  if (G.m < 32) issue_layer<LAYER>(sm, G);
   const bool ok = gsync_and(G.g, mbar_wait(G.bar_mma, G.ph_mma, err));
   if (ok) G.ph_mma ^= 1u;  // on a timeout the phase stays, so a final bounded wait watches the right one
   fence_after();
@@ -216,11 +223,11 @@ __device__ __forceinline__ void epilogue_to_tmem(const Group& G) {
 __device__ __forceinline__ float sigmoid_fast(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
 
 __device__ __forceinline__ bool mlp_tile(char* sm, Group& G, uint32_t* err, float c[3], bool folded_b1) {
-  if (!run_layer(sm, G, 0, err)) return false;
+  if (!run_layer<0>(sm, G, err)) return false;
   epilogue_hidden(G, folded_b1 ? nullptr : (const float*)(sm + Smem::b1));
-  if (!run_layer(sm, G, 1, err)) return false;
+  if (!run_layer<1>(sm, G, err)) return false;
   epilogue_to_tmem(G);
-  if (!run_layer(sm, G, 2, err)) return false;
+  if (!run_layer<2>(sm, G, err)) return false;
   float v[16];
   tmem_ld<16>(G.tmem + kL3Col + ((uint32_t)((G.m >> 5) * 32) << 16), v);
   const float* b3 = (const float*)(sm + Smem::b3);
@@ -514,15 +521,7 @@ __device__ __forceinline__ bool gather_tiles(char* sm, tc::Group& G, const GridG
     if (run) {
       // layer 1 of tile ti (its A was gathered in the previous iteration)
       gsync(G.g);
-      if (m == 0) {
-        fence_after();
-        const uint64_t da = smem_desc(smem_u32(G.act), 128u, kK2 * 16);
-        const uint64_t db = smem_desc(smem_u32(sm + Smem::w1), 128u, kK1 * 16);
-#pragma unroll
-        for (int s2 = 0; s2 < kK1 / 16; s2++)
-          mma_bf16(G.tmem, da + 16u * s2, db + 16u * s2, idesc_bf16(kHidden), s2 > 0 ? 1u : 0u);
-        mma_commit(G.bar_mma);
-      }
+      if (m < 32) issue_layer<0>(sm, G);
       mma_pending = true;
       // every thread is done with the staged brick: copy the next tile's brick if it differs
       if (STAGED && gather && (int)tg.z != loaded) {
@@ -538,19 +537,12 @@ __device__ __forceinline__ bool gather_tiles(char* sm, tc::Group& G, const GridG
       mma_pending = false;
       epilogue_hidden(G, in_dim < kK1 ? nullptr : (const float*)(sm + Smem::b1));
       mma_pending = true;
-      if (!(alive = run_layer(sm, G, 1, &w.hdr[0]))) break;
+      if (!(alive = run_layer<1>(sm, G, &w.hdr[0]))) break;
       mma_pending = false;
       epilogue_to_tmem(G);
       // layer 3 of tile ti, not waited for yet
       gsync(G.g);
-      if (m == 0) {
-        fence_after();
-        const uint64_t db = smem_desc(smem_u32(sm + Smem::w3), 128u, kHidden * 16);
-#pragma unroll
-        for (int s2 = 0; s2 < kHidden / 16; s2++)
-          mma_bf16_ta(G.tmem + kL3Col, G.tmem + 8u * s2, db + 16u * s2, idesc_bf16(kN3), s2 > 0 ? 1u : 0u);
-        mma_commit(G.bar_mma);
-      }
+      if (m < 32) issue_layer<2>(sm, G);
       mma_pending = true;
     }
     // payload of the tile after the one gathered now, and the descriptor after that
