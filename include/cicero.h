@@ -45,7 +45,9 @@ typedef enum {
 typedef enum { CICERO_F32 = 0, CICERO_F16 = 1 } cicero_dtype;
 
 /* Arithmetic of Feature Computation (the MLP):
- * FP32: FP32 FFMA on CUDA cores.  BF16: tcgen05 tensor-core MMAs with BF16 operands (weights and
+ * FP32: the accuracy of FP32.  cicero_mlp_eval runs FP32 FFMA on CUDA cores; the rendering calls split
+ * every operand of layers 1 and 2 into three BF16 parts (24 significand bits) and take the six products
+ * above 2^-24 on the tensor cores with FP32 accumulation; biases, layer 3 and the sigmoid in FP32.  BF16: tcgen05 tensor-core MMAs with BF16 operands (weights and
  * activations rounded to BF16) and FP32 accumulation in tensor memory.  FP32_SPLIT: FP32-class
  * accuracy on the tensor cores: every FP32 operand v of layers 1 and 2 is split into
  * hi = bf16(v) and lo = bf16(v - hi), each product taken as hi.hi + hi.lo + lo.hi (the method of
@@ -410,12 +412,13 @@ cicero_status cicero_warp_noalloc(const float *ref_rgb, const float *ref_depth,
  * [w1 [hidden][in_dim], b1 [hidden], w2 [hidden][hidden], b2 [hidden], w3 [3][hidden], b3 [3]]
  * (FP32, the layout of cicero_mlp's tensors back to back).  Gradients are summed with atomic adds,
  * so the order of the sums, and the last bits of the result, vary between calls.  Each ray's
- * forward pass is recomputed (nothing is stored by the forward).  Up to 16 feature channels the
- * recompute and the grid gradients run the MLP on the tensor cores with split-BF16 operands
- * (hi + lo, three products, FP32 accumulation), and the samples with a ReLU pre-activation within
- * an estimate of that precision's error of zero (~10 times the typical error) are recomputed in
- * FP32, so a mask differs from the FP32 MLP's only where the split products err by more than
- * that; wider grids recompute and differentiate in FP32 on the CUDA cores.  Early stop is a fixed
+ * forward pass is recomputed (nothing is stored by the forward).  The recompute runs the MLP on the
+ * tensor cores with operands of three BF16 parts (six products, FP32 accumulation).  Up to 16
+ * feature channels the samples with a ReLU pre-activation within an estimate of that precision's
+ * error of zero (~8 times the typical error) are recomputed in FP32 on the CUDA cores, so a mask
+ * differs from the FP32 MLP's only where the products err by more than that, and the grid gradients
+ * run on the tensor cores too (two parts, three products); wider grids differentiate in FP32 on the
+ * CUDA cores.  Early stop is a fixed
  * truncation.  For composited sample k:
  *   dL/dc_k = w_k g;  dL/dsigma_k = delta (T_{k+1} g.c_k - g.R_k), R_k = sum_{j>k} w_j c_j + T_end bg;
  *   dL/draw_k = dL/dsigma_k sigmoid(raw_k + shift); MLP chain rule; trilinear adjoint. */

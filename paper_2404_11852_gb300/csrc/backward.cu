@@ -2,10 +2,10 @@
 // feature grids.  Nothing is stored by the forward pass; the backward recomputes it:
 //
 //   forward recompute  K1-K4 of render.cu (march, Ray Index Table), then per brick the features
-//                      and the MLP: k_fwd_x3 (tensor cores, split-BF16 products) and k_fwd_fix
-//                      (FP32, the samples with a ReLU pre-activation within k_fwd_x3's error
-//                      estimate of zero); this
-//                      leaves per composited sample (c, w, T, raw density) and the ReLU masks
+//                      and the MLP: k_mlp_split (tensor cores, operands split into three BF16
+//                      parts) and k_fwd_fix (FP32 on the CUDA cores, the samples with a ReLU
+//                      pre-activation within k_mlp_split's error estimate of zero); this leaves
+//                      per composited sample (c, w, T, raw density) and the ReLU masks
 //   B1 k_bwd_ray       per ray (warp), in slot order: R_k = sum_{j>k} w_j c_j + T_end bg by a
 //                      warp scan, dL/dsigma_k = delta (T_{k+1} g.c_k - g.R_k) and
 //                      dL/draw_k = dL/dsigma_k * sigmoid(raw_k + shift); each record's colour
@@ -527,8 +527,8 @@ __global__ void __launch_bounds__(256, 1) k_bwd_brick(GridGeo g, RaySrc src, Mlp
 // lo = bf16(x - hi) and each product is hi hi' + hi lo' + lo hi' (the bf16x3 scheme of Henry, Tang
 // and Heinecke, ARITH 2019: the dropped lo lo' term and the residuals of the split are each ~2^-18
 // of the product, so a product keeps ~16 significant bits), accumulated in FP32 in tensor memory.
-// The ReLU masks are the recompute's (rec_mask): every decision whose pre-activation the split-BF16
-// recompute found within its error estimate of zero was taken again by the FP32 MLP.
+// The ReLU masks are the recompute's (rec_mask): every decision whose pre-activation it found within its
+// error estimate of zero was taken again by the FP32 MLP on the CUDA cores.
 
 namespace bt {
 constexpr int kGroups = 2;
@@ -608,16 +608,16 @@ __device__ __forceinline__ void stage_put(char* col, int op, int R, int g, const
   *reinterpret_cast<uint4*>(col + op + 32 * R + 256 * g) = lo;
 }
 
-// ReLU mask of the half h of the hidden units (h = 0: units 0..63, 1: 64..127), in the layout the
-// recompute writes (unit n < 64 is bit n % 4 of byte n / 4, unit 64 + n bit 4 + n % 4): the
-// words shifted so that unit 64 h + i is bit (i / 4 % 4) * 8 + i % 4 of word i / 16.
+// ReLU mask of the half h of the hidden units (h = 0: units 0..63, 1: 64..127), in the rec_mask layout
+// (words in the order 0, 2, 1, 3 of units 16 word ..): the words shifted so that unit 64 h + i is bit
+// (i / 4 % 4) * 8 + i % 4 of word i / 16.
 struct HalfMask {
   uint32_t w[4];
   __device__ __forceinline__ HalfMask(const uint4& mk, int h) {
     const uint32_t sh = 4u * (uint32_t)h;
     w[0] = mk.x >> sh;
-    w[1] = mk.y >> sh;
-    w[2] = mk.z >> sh;
+    w[1] = mk.z >> sh;
+    w[2] = mk.y >> sh;
     w[3] = mk.w >> sh;
   }
   __device__ __forceinline__ bool operator[](int i) const {  // i = 0..63, a compile-time constant in use
@@ -847,422 +847,6 @@ __global__ void __launch_bounds__(bt::kThreads, 1) k_bwd_brick_tc(GridGeo g, Mlp
   }
 }
 
-
-// ------------------------------------------------------------------------------------------------
-// The backward's forward recompute on the tensor cores.  Per tile of 128 samples of one brick:
-// x -> h1 = relu(W1 x + b1) -> h2 = relu(W2 h1 + b2) -> c = sigmoid(W3 h2 + b3), layers 1 and 2 as
-// tcgen05 MMAs on split-BF16 operands (hi + lo, three products per K step as in k_bwd_brick_tc,
-// FP32 accumulation in TMEM), the biases, layer 3 and the sigmoid in FP32 on the CUDA cores.  It
-// writes what the backward reads: (c, w) into rec_c and the ReLU masks of layers 1 and 2 into
-// rec_mask.  Two independent groups of 128 threads per CTA (alternate tiles, each its own operand
-// region, TMEM columns and mbarrier), one thread per sample: the thread interpolates its sample's
-// eight corners, stages its FP32 input row in shared memory (the row then read back in chunks), and
-// takes all 128 hidden units in the epilogues, 64 at a time.
-//
-// A ReLU decision taken on a split-BF16 pre-activation can differ from the FP32 one where the
-// pre-activation is within the products' error of zero, and one flipped mask moves that sample's
-// whole gradient through the unit.  So each decision is checked against an estimate of that
-// error: unit n of layer 1 is uncertain when |z1_n| <= eps ||W1_n|| ||x||, unit n of layer 2 when
-// |z2_n| <= eps ||W2_n|| (||h1|| + ||x|| ||W1||_F) (its own products plus layer 1's errors carried
-// through W2).  Each split product drops terms of at most ~3 2^-18 |w x|, and the rounding errors
-// of a K-term sum add up like a random walk, to ~2^-17 ||w o x||_2, while ||w|| ||x|| is about
-// sqrt(K) ||w o x||_2: eps = 2^-17 leaves a margin of 7 to 11 times the typical error (K = 48,
-// 128).  The samples with an uncertain decision are listed (their sorted record index, in rec_key,
-// which the Ray Index Table no longer needs; count in hdr[4]) and recomputed by the FP32 MLP
-// afterwards (k_fwd_fix), so their masks are the FP32 path's.  On the 8192-ray workload 8.6% of
-// the samples are listed (16.5% with eps = 2^-16, 4.4% with 2^-18; the gradients of the three
-// parity scenes agree with the FP64 oracle to ~5e-6 in all three cases, and to 2e-3 without the
-// fix-up).
-namespace xt {
-constexpr int kGroups = 2;
-constexpr int kThreads = kGroups * kTile;  // one thread per sample of each group's 128-sample tile
-constexpr int kK1 = 48;                    // layer-1 K: in_dim padded to a multiple of 16
-constexpr int kMaxC = 16;                  // feature channels
-constexpr int kXS = kK1 + 1;               // FP32 row stride of the staged inputs (odd: rows in distinct banks)
-constexpr float kEps = 7.62939453125e-06f;  // 2^-17
-// A group's operand region (64 KB).  While x is built: the FP32 rows at [0, 128 kXS 4) and the
-// layer-1 operand x (hi, lo; K = 48) at [40 KB, 64 KB).  From layer 1's epilogue on: h1 hi at
-// [0, 32 KB), lo at [32 KB, 64 KB), written once layer 1's MMA has read x and every row was read.
-struct Region {
-  static constexpr int xs = 0;
-  static constexpr int x_hi = 40 * 1024;
-  static constexpr int x_lo = x_hi + kTile * kK1 * 2;
-  static constexpr int h_hi = 0;
-  static constexpr int h_lo = kTile * kHidden * 2;
-  static constexpr int bytes = 2 * kTile * kHidden * 2;
-  static_assert(xs + kTile * kXS * 4 <= x_hi && x_lo + kTile * kK1 * 2 == bytes, "region layout");
-};
-struct Smem {
-  static constexpr int w1_hi = 0;                             // [128][48] bf16: row n, K = k: W1[n][k]
-  static constexpr int w1_lo = w1_hi + kHidden * kK1 * 2;
-  static constexpr int w2_hi = w1_lo + kHidden * kK1 * 2;     // [128][128] bf16: row n, K = k: W2[n][k]
-  static constexpr int w2_lo = w2_hi + kHidden * kHidden * 2;
-  static constexpr int region = w2_lo + kHidden * kHidden * 2;  // kGroups operand regions
-  static constexpr int prm = region + kGroups * Region::bytes;  // b1 [128], b2 [128], w3 [3][128], b3 [4] f32
-  static constexpr int nrm = prm + (5 * kHidden + 4) * 4;     // ||W1_n|| [128], ||W2_n|| [128], ||W1||_F f32
-  static constexpr int bars = nrm + (2 * kHidden + 4) * 4;    // one mbarrier per group; TMEM address at +16
-  static constexpr int bytes = bars + 128;
-  static_assert(region % 16 == 0 && w2_hi % 16 == 0 && bars % 16 == 0, "alignment");
-};
-constexpr uint32_t kTmemCols = kGroups * 128;  // 128 columns per group
-}  // namespace xt
-
-bool fwd_x3_supported(const GridGeo& g, const MlpPtrs& mlp) {
-  return g.C <= xt::kMaxC && mlp.in_dim <= xt::kK1 && mlp.in_dim == g.C + 3 + 6 * mlp.n_freq;
-}
-
-// Bits of this thread's ReLU decisions: unit 64 h + n (n < 64) is bit ((n / 4) % 4) * 8 + 4 h + n % 4
-// of word n / 16 (the rec_mask layout)
-__device__ __forceinline__ void relu_bit(uint32_t mw[4], int n, int h, bool on) {
-  mw[n >> 4] |= (on ? 1u : 0u) << (((n >> 2) & 3) * 8 + 4 * h + (n & 3));
-}
-
-// BWD: the backward's recompute (masks, uncertain samples listed); otherwise a forward render's
-// Feature Computation (colours only).  WG (with BWD): also stage x, h1 and h2 for the weight gradients.
-template <typename T, bool BWD, bool WG = false>
-__global__ void __launch_bounds__(xt::kThreads, 1) k_fwd_x3(GridGeo g, MlpPtrs mlp, RenderWs w,
-                                                            const T* __restrict__ feat) {
-  using namespace tc;
-  extern __shared__ __align__(1024) char sm[];
-  const int C = g.C, B = g.brick;
-  const int m = threadIdx.x & (kTile - 1), grp = threadIdx.x / kTile;
-  char* region = sm + xt::Smem::region + grp * xt::Region::bytes;
-  char* h_hi = region + xt::Region::h_hi;
-  char* h_lo = region + xt::Region::h_lo;
-  float* xs = (float*)(region + xt::Region::xs) + m * xt::kXS;  // this sample's FP32 row
-  float* b1s = (float*)(sm + xt::Smem::prm);
-  float* b2s = b1s + kHidden;
-  float* w3s = b2s + kHidden;
-  float* b3s = w3s + 3 * kHidden;
-  float* nw1 = (float*)(sm + xt::Smem::nrm);
-  float* nw2 = nw1 + kHidden;
-  float* fro1 = nw2 + kHidden;
-  uint64_t* bar = (uint64_t*)(sm + xt::Smem::bars) + grp;
-  uint32_t* tslot = (uint32_t*)(sm + xt::Smem::bars + 16);
-  // the weights, split into the hi and lo B operands; the other parameters in FP32
-  for (int i = threadIdx.x; i < kHidden * (xt::kK1 / 8); i += xt::kThreads) {
-    const int n = i / (xt::kK1 / 8), k0 = (i % (xt::kK1 / 8)) * 8;
-    float v[8];
-#pragma unroll
-    for (int j = 0; j < 8; j++) v[j] = k0 + j < mlp.in_dim ? mlp.w1[n * mlp.in_dim + k0 + j] : 0.0f;
-    store_chunk_split(sm + xt::Smem::w1_hi, sm + xt::Smem::w1_lo, n, k0, xt::kK1, v);
-  }
-  for (int i = threadIdx.x; i < kHidden * (kHidden / 8); i += xt::kThreads) {
-    const int n = i / (kHidden / 8), k0 = (i % (kHidden / 8)) * 8;
-    float v[8];
-#pragma unroll
-    for (int j = 0; j < 8; j++) v[j] = mlp.w2[n * kHidden + k0 + j];
-    store_chunk_split(sm + xt::Smem::w2_hi, sm + xt::Smem::w2_lo, n, k0, kHidden, v);
-  }
-  for (int i = threadIdx.x; i < kHidden; i += xt::kThreads) {
-    b1s[i] = mlp.b1[i];
-    b2s[i] = mlp.b2[i];
-  }
-  for (int i = threadIdx.x; i < 3 * kHidden; i += xt::kThreads) w3s[i] = mlp.w3[i];
-  if (threadIdx.x < 4) b3s[threadIdx.x] = threadIdx.x < 3 ? mlp.b3[threadIdx.x] : 0.0f;
-  if constexpr (BWD) {  // row norms of W1 (threads < 128) and W2 (the others)
-    const int n = threadIdx.x & (kHidden - 1);
-    float s2 = 0.0f;
-    if (threadIdx.x < kHidden)
-      for (int k = 0; k < mlp.in_dim; k++) s2 = fmaf(mlp.w1[n * mlp.in_dim + k], mlp.w1[n * mlp.in_dim + k], s2);
-    else
-      for (int k = 0; k < kHidden; k++) s2 = fmaf(mlp.w2[n * kHidden + k], mlp.w2[n * kHidden + k], s2);
-    (threadIdx.x < kHidden ? nw1 : nw2)[n] = sqrtf(s2);
-  }
-  if (threadIdx.x == 0) {
-    for (int j = 0; j < xt::kGroups; j++) mbar_init((uint64_t*)(sm + xt::Smem::bars) + j, 1);
-    fence_mbar_init();
-  }
-  fence_proxy_async();
-  if (threadIdx.x < 32) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                 "r"(xt::kTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  fence_before();
-  __syncthreads();
-  fence_after();
-  if (BWD && threadIdx.x == 0) {  // read after the first tile's first group barrier
-    float f2 = 0.0f;
-    for (int n = 0; n < kHidden; n++) f2 = fmaf(nw1[n], nw1[n], f2);
-    *fro1 = sqrtf(f2);
-  }
-  __syncthreads();
-  const uint32_t tmem_base = *tslot;
-  const uint32_t tmem = tmem_base + 128u * (uint32_t)grp;                             // this group's columns
-  const uint32_t taddr = tmem + ((uint32_t)(((threadIdx.x >> 5) & 3) * 32) << 16);  // this warp's lanes
-  const uint64_t ax_h = smem_desc(smem_u32(region + xt::Region::x_hi), 128u, xt::kK1 * 16);
-  const uint64_t ax_l = smem_desc(smem_u32(region + xt::Region::x_lo), 128u, xt::kK1 * 16);
-  const uint64_t ah_h = smem_desc(smem_u32(h_hi), 128u, kHidden * 16), ah_l = smem_desc(smem_u32(h_lo), 128u, kHidden * 16);
-  const uint64_t b1h = smem_desc(smem_u32(sm + xt::Smem::w1_hi), 128u, xt::kK1 * 16);
-  const uint64_t b1l = smem_desc(smem_u32(sm + xt::Smem::w1_lo), 128u, xt::kK1 * 16);
-  const uint64_t b2h = smem_desc(smem_u32(sm + xt::Smem::w2_hi), 128u, kHidden * 16);
-  const uint64_t b2l = smem_desc(smem_u32(sm + xt::Smem::w2_lo), 128u, kHidden * 16);
-  const int ne = 3 + 6 * mlp.n_freq;
-  uint32_t phase = 0;
-  bool alive = true;
-
-  const uint32_t n_tiles = w.hdr[1];
-  const uint32_t per = (n_tiles + gridDim.x - 1) / gridDim.x;
-  const uint32_t t_begin = blockIdx.x * per, t_end = min(n_tiles, t_begin + per);
-  // this thread's sorted record of the group's next tile, loaded when the current tile starts
-  uint4 n_td = make_uint4(0u, 0u, 0u, 0u);
-  float4 n_pw = make_float4(0.f, 0.f, 0.f, 0.f), n_qd = n_pw;
-  auto prefetch = [&](uint32_t t) {
-    n_td = w.tile[t];
-    if (m < (int)(n_td.y & 0xFFu)) {
-      n_pw = w.srt[n_td.x + m].pw;
-      n_qd = w.srt[n_td.x + m].qd;
-    }
-  };
-  if (t_begin + grp < t_end) prefetch(t_begin + grp);
-  for (uint32_t ti = t_begin + grp; ti < t_end && alive; ti += xt::kGroups) {
-    const uint4 td = n_td;
-    const float4 pw = n_pw, qd = n_qd;
-    if (ti + xt::kGroups < t_end) prefetch(ti + xt::kGroups);
-    const uint32_t start = td.x;
-    const int mcnt = (int)(td.y & 0xFFu);
-    const int bx = (int)(td.w & 0xFFFFu), by = (int)(td.w >> 16), bz = (int)((td.y >> 8) & 0x1FFFu);
-    const bool valid = m < mcnt;
-    // the weight gradients' operands of this sample (backward with d_mlp): column start + m
-    char* stg = (BWD && WG && valid) ? w.stage + stage_col(start + m) : nullptr;
-    uint32_t rid = 0;
-    float wgt = 0.0f, fx[xt::kMaxC];
-#pragma unroll
-    for (int c = 0; c < xt::kMaxC; c++) fx[c] = 0.0f;
-    if (valid) {
-      rid = __float_as_uint(qd.x);
-      wgt = pw.w;
-      const float p[3] = {pw.x, pw.y, pw.z};
-      int i0[3];
-      float f[3];
-      const bool in = index_sample(g, p, i0, f);
-      const int l[3] = {i0[0] - bx * B, i0[1] - by * B, i0[2] - bz * B};
-      if (!(in && l[0] >= 0 && l[0] < B && l[1] >= 0 && l[1] < B && l[2] >= 0 && l[2] < B)) {
-        set_err(&w.hdr[0], kErrInternal);
-      } else {
-#pragma unroll
-        for (int q = 0; q < 8; q++) {
-          const float wq = corner_weight(f[0], f[1], f[2], q);
-          const T* v = feat + corner_vertex(g, i0[0], i0[1], i0[2], q) * (size_t)C;
-#pragma unroll
-          for (int c = 0; c < xt::kMaxC; c++)
-            if (c < C) fx[c] = fmaf(wq, ldf(v + c), fx[c]);
-        }
-      }
-    }
-    // this sample's FP32 row of x (features, direction encoding, zeros), staged, then split into
-    // the layer-1 operand 8 K values at a time
-#pragma unroll
-    for (int c = 0; c < xt::kMaxC; c++)
-      if (c < C) xs[c] = fx[c];
-    if (valid) {
-      const float d[3] = {qd.y, qd.z, qd.w};
-      encode_dir(d, mlp.n_freq, xs + C);
-    } else {
-      for (int j = 0; j < ne; j++) xs[C + j] = 0.0f;
-    }
-    for (int k = C + ne; k < xt::kK1; k++) xs[k] = 0.0f;
-    float x2 = 0.0f;
-#pragma unroll
-    for (int j = 0; j < xt::kK1 / 8; j++) {
-      float v[8];
-#pragma unroll
-      for (int t = 0; t < 8; t++) {
-        v[t] = xs[8 * j + t];
-        x2 = fmaf(v[t], v[t], x2);
-      }
-      uint4 hi, lo;
-      split8(v, hi, lo);
-      store_rows(region + xt::Region::x_hi, region + xt::Region::x_lo, m, 8 * j, xt::kK1, hi, lo);
-      if (WG && stg) stage_put(stg, WgStage::x, xt::kK1, j, hi, lo);
-    }
-    fence_proxy_async();
-    fence_before();
-    group_sync(grp);
-    // layer 1: W1 x into the group's columns [0, 128)
-    if (m == 0) {
-      fence_after();
-      mma_split<xt::kK1 / 16>(tmem, ax_h, ax_l, b1h, b1l, idesc_bf16(kHidden));
-      mma_commit(bar);
-    }
-    alive = group_sync_and(grp, mbar_wait(bar, phase, &w.hdr[0]));
-    fence_after();
-    if (!alive) break;
-    phase ^= 1u;
-    uint32_t mw1[4] = {0u, 0u, 0u, 0u}, mw2[4] = {0u, 0u, 0u, 0u};
-    const float tx = xt::kEps * sqrtf(x2);
-    bool unsure = false;
-    float h2s = 0.0f;  // ||h1||^2
-#pragma unroll 1
-    for (int h = 0; h < 2; h++) {
-      float v[64];
-      tmem_ld<64>(taddr + 64 * h, v);
-      const float4* b4 = reinterpret_cast<const float4*>(b1s + 64 * h);  // per-unit constants, 4 at a time
-      const float4* n4 = reinterpret_cast<const float4*>(nw1 + 64 * h);
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        float x[8];
-#pragma unroll
-        for (int t4 = 0; t4 < 2; t4++) {
-          const float4 bq = b4[2 * q + t4];
-          const float bv[4] = {bq.x, bq.y, bq.z, bq.w};
-          float nv[4] = {0.f, 0.f, 0.f, 0.f};
-          if constexpr (BWD) {
-            const float4 nq = n4[2 * q + t4];
-            nv[0] = nq.x;
-            nv[1] = nq.y;
-            nv[2] = nq.z;
-            nv[3] = nq.w;
-          }
-#pragma unroll
-          for (int j = 0; j < 4; j++) {
-            const int t = 4 * t4 + j, n = 8 * q + t;
-            const float z = v[n] + bv[j];
-            if constexpr (BWD) {
-              relu_bit(mw1, n, h, z > 0.0f);
-              unsure |= fabsf(z) <= tx * nv[j];
-            }
-            x[t] = fmaxf(z, 0.0f);
-            h2s = fmaf(x[t], x[t], h2s);
-          }
-        }
-        uint4 hi, lo;
-        split8(x, hi, lo);
-        store_rows(h_hi, h_lo, m, 64 * h + 8 * q, kHidden, hi, lo);
-        if (WG && stg) stage_put(stg, WgStage::h1, kHidden, 8 * h + q, hi, lo);
-      }
-    }
-    fence_proxy_async();
-    fence_before();
-    group_sync(grp);
-    // layer 2: W2 h1 into the group's columns [0, 128)
-    if (m == 0) {
-      fence_after();
-      mma_split(tmem, ah_h, ah_l, b2h, b2l, idesc_bf16(kHidden));
-      mma_commit(bar);
-    }
-    alive = group_sync_and(grp, mbar_wait(bar, phase, &w.hdr[0]));
-    fence_after();
-    if (!alive) break;
-    phase ^= 1u;
-    float z0 = 0.0f, z1 = 0.0f, z2 = 0.0f;
-    float h2v[8];  // h2 of 8 consecutive units, staged once complete (WG)
-    const float th = BWD ? xt::kEps * (sqrtf(h2s) + sqrtf(x2) * *fro1) : 0.0f;
-#pragma unroll 1
-    for (int h = 0; h < 2; h++) {
-      float v[64];
-      tmem_ld<64>(taddr + 64 * h, v);
-      const float4* b4 = reinterpret_cast<const float4*>(b2s + 64 * h);  // per-unit constants, 4 at a time
-      const float4* n4 = reinterpret_cast<const float4*>(nw2 + 64 * h);
-      const float4* w0 = reinterpret_cast<const float4*>(w3s + 64 * h);
-      const float4* w1 = reinterpret_cast<const float4*>(w3s + kHidden + 64 * h);
-      const float4* w2 = reinterpret_cast<const float4*>(w3s + 2 * kHidden + 64 * h);
-#pragma unroll
-      for (int n4i = 0; n4i < 16; n4i++) {
-        const float4 bq = b4[n4i], c0 = w0[n4i], c1 = w1[n4i], c2 = w2[n4i];
-        const float bv[4] = {bq.x, bq.y, bq.z, bq.w};
-        const float u0[4] = {c0.x, c0.y, c0.z, c0.w}, u1[4] = {c1.x, c1.y, c1.z, c1.w}, u2[4] = {c2.x, c2.y, c2.z, c2.w};
-        float nv[4] = {0.f, 0.f, 0.f, 0.f};
-        if constexpr (BWD) {
-          const float4 nq = n4[n4i];
-          nv[0] = nq.x;
-          nv[1] = nq.y;
-          nv[2] = nq.z;
-          nv[3] = nq.w;
-        }
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-          const int n = 4 * n4i + j;
-          const float z = v[n] + bv[j];
-          if constexpr (BWD) {
-            relu_bit(mw2, n, h, z > 0.0f);
-            unsure |= fabsf(z) <= th * nv[j];
-          }
-          const float a2 = fmaxf(z, 0.0f);
-          if constexpr (WG) h2v[4 * (n4i & 1) + j] = a2;
-          z0 = fmaf(u0[j], a2, z0);
-          z1 = fmaf(u1[j], a2, z1);
-          z2 = fmaf(u2[j], a2, z2);
-        }
-        if (WG && stg && (n4i & 1)) {  // units 64 h + 8 (n4i / 2) .. + 7 complete
-          uint4 hi, lo;
-          split8(h2v, hi, lo);
-          stage_put(stg, WgStage::h2, kHidden, 8 * h + n4i / 2, hi, lo);
-        }
-      }
-    }
-    fence_before();
-    if constexpr (BWD) {  // list the uncertain samples (one atomic per warp)
-      const bool fix = valid && unsure;
-      const uint32_t bal = __ballot_sync(0xffffffffu, fix);
-      uint32_t base = 0;
-      if ((threadIdx.x & 31) == 0 && bal) base = atomicAdd(&w.hdr[4], (uint32_t)__popc(bal));
-      base = __shfl_sync(0xffffffffu, base, 0);
-      if (fix) w.rec_key[base + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u))] = start + m;
-    }
-    if (valid) {
-      w.rec_c[rid] = make_float4(sigmoid_f(z0 + b3s[0]), sigmoid_f(z1 + b3s[1]), sigmoid_f(z2 + b3s[2]), wgt);
-      if constexpr (BWD) {
-        w.rec_mask[2 * (size_t)rid] = make_uint4(mw1[0], mw1[1], mw1[2], mw1[3]);
-        w.rec_mask[2 * (size_t)rid + 1] = make_uint4(mw2[0], mw2[1], mw2[2], mw2[3]);
-      }
-    }
-  }
-  if (!alive) mbar_wait(bar, phase, &w.hdr[0]);  // MMAs may still be running (bounded)
-  fence_before();
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(xt::kTmemCols)
-                 : "memory");
-  }
-}
-
-cicero_status launch_fwd_x3(const cicero_grid* grid, const GridGeo& geo, const MlpPtrs& mlp, const RenderWs& ws,
-                            cudaStream_t st) {
-  const bool f16 = grid->dtype == CICERO_F16, bwd = ws.rec_mask != nullptr;
-  cudaError_t e = cudaSuccess;
-  const int sb = xt::Smem::bytes;
-  const dim3 grid_dim(num_sms()), block(xt::kThreads);
-  {
-    ProfScope ps(kStGatherMlp, st);
-    if (bwd && ws.stage) {  // the backward with the weight gradients' staging
-      if (f16) {
-        e = cudaFuncSetAttribute(k_fwd_x3<__half, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb);
-        if (e == cudaSuccess)
-          k_fwd_x3<__half, true, true><<<grid_dim, block, sb, st>>>(geo, mlp, ws, (const __half*)grid->features);
-      } else {
-        e = cudaFuncSetAttribute(k_fwd_x3<float, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb);
-        if (e == cudaSuccess)
-          k_fwd_x3<float, true, true><<<grid_dim, block, sb, st>>>(geo, mlp, ws, (const float*)grid->features);
-      }
-    } else if (f16) {
-      const __half* feat = (const __half*)grid->features;
-      if (bwd) {
-        e = cudaFuncSetAttribute(k_fwd_x3<__half, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb);
-        if (e == cudaSuccess) k_fwd_x3<__half, true><<<grid_dim, block, sb, st>>>(geo, mlp, ws, feat);
-      } else {
-        e = cudaFuncSetAttribute(k_fwd_x3<__half, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb);
-        if (e == cudaSuccess) k_fwd_x3<__half, false><<<grid_dim, block, sb, st>>>(geo, mlp, ws, feat);
-      }
-    } else {
-      const float* feat = (const float*)grid->features;
-      if (bwd) {
-        e = cudaFuncSetAttribute(k_fwd_x3<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb);
-        if (e == cudaSuccess) k_fwd_x3<float, true><<<grid_dim, block, sb, st>>>(geo, mlp, ws, feat);
-      } else {
-        e = cudaFuncSetAttribute(k_fwd_x3<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb);
-        if (e == cudaSuccess) k_fwd_x3<float, false><<<grid_dim, block, sb, st>>>(geo, mlp, ws, feat);
-      }
-    }
-  }
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_fwd_x3)");
-  count_launches(1);
-  e = cudaGetLastError();
-  return e == cudaSuccess ? CICERO_OK : cuda_fail(e, "k_fwd_x3");
-}
 
 // ------------------------------------------------------------------------------------------------
 // The MLP weight gradients on the tensor cores, from the operands that the recompute (x, h1, h2)
@@ -1498,6 +1082,8 @@ static cudaError_t launch_bwd_brick(const RenderPlan& plan, const RaySrc& src, c
   return cudaGetLastError();
 }
 
+bool tc_backward(const GridGeo& g) { return g.C <= bt::kN1; }
+
 cicero_status run_backward(const cicero_grid* grid, const MlpPtrs& mlp, const RenderPlan& plan, const RaySrc& src,
                            const RenderWs& ws, const float* d_rgb, float* d_dens, float* d_feat, float* d_mlp,
                            cudaStream_t st) {
@@ -1517,7 +1103,7 @@ cicero_status run_backward(const cicero_grid* grid, const MlpPtrs& mlp, const Re
   const bool f16 = grid->dtype == CICERO_F16;
   cudaError_t e;
   const int smem_tc = bt::Smem::bytes;
-  if (ws.rec_mask && plan.geo.C <= bt::kN1 && (!d_mlp || ws.stage)) {
+  if (tc_backward(plan.geo) && (!d_mlp || ws.stage)) {
     // grid gradients on the tensor cores, with the recompute's ReLU masks; with d_mlp, the weight
     // gradients' operands staged on the way and the weight gradients as tensor-core GEMMs after
     {

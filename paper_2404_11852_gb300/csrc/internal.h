@@ -64,8 +64,9 @@ struct RenderWs {
   float* rec_T;         // [Q] transmittance before the slot (backward only; may be null)
   float* rec_raw;       // [Q] interpolated raw density (backward only; may be null)
   uint32_t* rec_ray;    // [Q] ray of each record (RIT export only; may be null)
-  uint4* rec_mask;      // [Q][2] ReLU masks of MLP layers 1 and 2 from the FP32 forward (backward only; may be
-                        // null): hidden unit n < 64 is bit n % 4 of byte n / 4, unit 64 + n is bit 4 + n % 4
+  uint4* rec_mask;      // [Q][2] ReLU masks of MLP layers 1 and 2 from the recompute (backward only; may be
+                        // null): hidden unit n < 64 is bit n % 4 of byte n / 4 % 4 of word n / 16, unit 64 + n
+                        // the bit 4 above it; the words stand in the order 0, 2, 1, 3
   uint32_t* brick_cnt;  // [nb * kOctants] records per RIT key
   uint32_t* brick_off;  // [nb * kOctants + 1] first record of each key (brick b starts at key b * kOctants)
   uint32_t* brick_cur;  // [nb * kOctants] scatter cursors
@@ -224,6 +225,10 @@ cicero_status launch_mlp_eval_bf16(const MlpPtrs& mlp, const float* x, int M, fl
 // (mlp_split.cu)
 cicero_status launch_mlp_split(const cicero_grid* grid, const GridGeo& geo, int parts, const MlpPtrs& mlp,
                                const RenderWs& ws, cudaStream_t st);
+// the backward's forward recompute, three parts: (c, w) into rec_c and the ReLU masks into rec_mask, the
+// samples with an uncertain decision listed; with ws.stage also the weight gradients' operands x, h1 and h2
+cicero_status launch_mlp_recompute(const cicero_grid* grid, const GridGeo& geo, const MlpPtrs& mlp, const RenderWs& ws,
+                                   cudaStream_t st);
 
 // SpaRW warp (warp.cu)
 struct WarpArgs {
@@ -273,12 +278,9 @@ cicero_status run_backward(const cicero_grid* grid, const MlpPtrs& mlp, const Re
                            cudaStream_t st);
 cicero_status launch_mlp_eval_f32(const MlpPtrs& mlp, const float* x, int M, float* c, cudaStream_t st);
 
-// The backward's forward recompute on the tensor cores (split-BF16 products, FP32 accumulation):
-// (c, w) into rec_c and the ReLU masks into rec_mask for every composited sample (backward.cu)
-bool fwd_x3_supported(const GridGeo& g, const MlpPtrs& mlp);
+// whether the backward's tensor-core kernels take the grid (up to 16 channels)
+bool tc_backward(const GridGeo& g);
 // dW1 | db1, dW2 | db2, dW3 (and db3) from the staged operands, added to d_mlp (backward.cu)
 cicero_status launch_dw(const MlpPtrs& mlp, const RenderWs& ws, float* d_mlp, cudaStream_t st);
-cicero_status launch_fwd_x3(const cicero_grid* grid, const GridGeo& geo, const MlpPtrs& mlp, const RenderWs& ws,
-                            cudaStream_t st);
 
 }  // namespace cicero

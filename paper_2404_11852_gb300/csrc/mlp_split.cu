@@ -45,16 +45,16 @@ constexpr int kEpiWarps = 8, kGatWarps = 4;  // warps of E1 and of E2; warps of 
 constexpr int kE2 = kEpiWarps, kG = 2 * kEpiWarps, kM = kG + 2 * kGatWarps;  // first warp of each role
 constexpr int kThreads = 32 * (kM + 4);      // M's warpgroup has one working warp
 // Registers per thread: 72 at launch (28 warps), then shared out by role (setmaxnreg):
-// 256 (88 + 80 + 72) + 128 x 24 = 896 x 72.
-constexpr int kRegsE1 = 88, kRegsE2 = 80, kRegsG = 72, kRegsM = 24;
-static_assert(kThreads == 896 && 256 * (kRegsE1 + kRegsE2 + kRegsG) + 128 * kRegsM <= kThreads * 72, "register shares");
+// 256 (E1 + E2 + G) + 128 x 24 = 896 x 72.  HOLD: see k_mlp_split.
+template <bool HOLD>
+struct Regs {
+  static constexpr int e1 = HOLD ? 88 : 72, e2 = HOLD ? 80 : 72, g = HOLD ? 72 : 96, m = 24;
+  static_assert(kThreads == 896 && 256 * (e1 + e2 + g) + 128 * m <= kThreads * 72, "register shares");
+};
 template <int R>
-__device__ __forceinline__ void regs_up() {
-  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R));
-}
-template <int R>
-__device__ __forceinline__ void regs_down() {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R));
+__device__ __forceinline__ void set_regs() {
+  if constexpr (R > 72) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R));
+  if constexpr (R < 72) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R));
 }
 constexpr int kChunks = 2;                  // chunks of hidden units of layer 2's K
 constexpr int kMeta = 4;                    // tiles of per-sample data in flight
@@ -70,10 +70,15 @@ struct Smem {
   static constexpr int l3 = b1 + kHidden * 4;                // per pair of hidden units: b2, w3 rows 0, 1, 2
   static constexpr int b3 = l3 + 4 * kHidden * 4;            // [4]
   static constexpr int z = b3 + 16;                          // [kMeta][128] float4: partial layer-3 sums
-  static constexpr int meta = z + kMeta * kTile * 16;        // [kMeta][128] float4: record, weight
+  static constexpr int meta = z + kMeta * kTile * 16;        // [kMeta][128] float4: record, weight, sorted place, ||x||^2
   static constexpr int bars = meta + kMeta * kTile * 16;
   static constexpr int bytes = bars + 8 * 32;
-  static_assert(x % 16 == 0 && w2 % 16 == 0 && bars % 16 == 0 && bytes <= 227 * 1024, "layout");
+  // a backward's recompute: ||W1_n|| [128], ||W2_n|| [128], ||W1||_F, then [2][2][128]: partial ||h1||^2 of
+  // two tiles, by half of the hidden units, the sign bit set where a decision is uncertain
+  static constexpr int nrm = bytes;
+  static constexpr int hs = nrm + (2 * kHidden + 4) * 4;
+  static constexpr int bytes_bwd = hs + 2 * 2 * kTile * 4;
+  static_assert(x % 16 == 0 && w2 % 16 == 0 && bars % 16 == 0 && bytes_bwd <= 227 * 1024, "layout");
 };
 
 struct Bars {  // one phase per use, in tile order
@@ -85,6 +90,7 @@ struct Bars {  // one phase per use, in tile order
   uint64_t dfree[2];       // accumulator of tile i read                   (8 E2 warps)
   uint64_t zfull[kMeta];   // partial layer-3 sums of tile i written       (4 E2 warps)
   uint64_t mfull[kMeta];   // per-sample data of tile i written            (4 G warps)
+  uint64_t hfull[2];       // partial ||h1||^2 of tile i written           (8 E1 warps, backward)
   uint64_t last;           // every MMA done                               (commit)
   uint32_t tmem;
 };
@@ -124,6 +130,24 @@ __device__ __forceinline__ void load_half(uint32_t d, int h, float* v) {
       : "memory");
 #pragma unroll
   for (int i = 0; i < 64; i++) v[i] = __uint_as_float(r[i]);
+}
+
+// Columns 32 c + 16 h + j (c = 2 g, 2 g + 1, j < 16) of this thread's lane of the accumulator at d.
+__device__ __forceinline__ void load_quarter(uint32_t d, int h, int g, float* v) {
+  uint32_t r[32];
+  const uint32_t a = d + 16u * (uint32_t)h + 64u * (uint32_t)g;
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(a), "r"(a + 32u)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]);
 }
 
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
@@ -229,25 +253,36 @@ __device__ __forceinline__ void gather(const GridGeo& g, const T* __restrict__ f
                                        float* out) {
   const int C = CC ? CC : g.C;
   constexpr int N = CC ? CC : kMaxC;
+  float wq[8];
+  const T* v[4];  // the x-pairs of vertices: (y, z) = (0, 0), (1, 0), (0, 1), (1, 1)
 #pragma unroll
-  for (int q = 0; q < 8; q++) {
-    const float wq = ((q & 1) ? f[0] : 1.f - f[0]) * (((q >> 1) & 1) ? f[1] : 1.f - f[1]) * ((q >> 2) ? f[2] : 1.f - f[2]);
-    const T* v = feat + (((size_t)(i0[2] + (q >> 2)) * g.n[1] + (i0[1] + ((q >> 1) & 1))) * g.n[0] + (i0[0] + (q & 1))) * C;
-    if (CC ? CC % 4 == 0 : (C & 3) == 0) {  // rows of the grid start on 16 bytes, vertices on 4 channels
+  for (int q = 0; q < 8; q++)
+    wq[q] = ((q & 1) ? f[0] : 1.f - f[0]) * (((q >> 1) & 1) ? f[1] : 1.f - f[1]) * ((q >> 2) ? f[2] : 1.f - f[2]);
 #pragma unroll
-      for (int c = 0; c + 4 <= N; c += 4)
-        if (CC || c < C) {
-          const float4 a = ld4(v + c);
-          out[c] = fmaf(wq, a.x, out[c]);
-          out[c + 1] = fmaf(wq, a.y, out[c + 1]);
-          out[c + 2] = fmaf(wq, a.z, out[c + 2]);
-          out[c + 3] = fmaf(wq, a.w, out[c + 3]);
+  for (int r = 0; r < 4; r++)
+    v[r] = feat + (((size_t)(i0[2] + (r >> 1)) * g.n[1] + (i0[1] + (r & 1))) * g.n[0] + i0[0]) * C;
+  if (CC ? CC % 4 == 0 : (C & 3) == 0) {  // rows of the grid start on 16 bytes, vertices on 4 channels
+#pragma unroll
+    for (int c = 0; c + 4 <= N; c += 4)
+      if (CC || c < C) {  // the eight corners' loads of four channels in flight together
+        float4 a[8];
+#pragma unroll
+        for (int q = 0; q < 8; q++) a[q] = ld4(v[q >> 1] + (q & 1) * C + c);
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+          out[c] = fmaf(wq[q], a[q].x, out[c]);
+          out[c + 1] = fmaf(wq[q], a[q].y, out[c + 1]);
+          out[c + 2] = fmaf(wq[q], a[q].z, out[c + 2]);
+          out[c + 3] = fmaf(wq[q], a[q].w, out[c + 3]);
         }
-    } else {
+      }
+  } else {
 #pragma unroll
-      for (int c = 0; c < N; c++)
-        if (c < C) out[c] = fmaf(wq, ldf(v + c), out[c]);
-    }
+    for (int c = 0; c < N; c++)
+      if (c < C) {
+#pragma unroll
+        for (int q = 0; q < 8; q++) out[c] = fmaf(wq[q], ldf(v[q >> 1] + (q & 1) * C + c), out[c]);
+      }
   }
 }
 
@@ -276,7 +311,7 @@ __device__ __forceinline__ void encode(const float d[3], float* x) {
 // M: every MMA of the CTA's n tiles, by one warp: the control flow and the operands are the warp's, one
 // elected lane issues.  (Issued from a thread of its own, each MMA's operands took a dozen instructions
 // through per-thread registers: ~110 clocks an MMA beside 27 other warps, against the 64 it runs.)
-template <int NP>
+template <int NP, bool HOLD>
 __device__ __forceinline__ void issue_mmas(char* sm, Bars& B, uint32_t tmem, uint32_t n, uint32_t* err) {
   using namespace tc;
   using S = Smem<NP>;
@@ -314,7 +349,7 @@ __device__ __forceinline__ void issue_mmas(char* sm, Bars& B, uint32_t tmem, uin
 #pragma unroll
     for (int c = 0; c < kChunks; c++) {
       if (c == kChunks / 2 && i + 1 < n && !(alive = layer1(i + 1))) break;
-      if (!(alive = warp_wait(&B.afull[c], i & 1, err))) break;
+      if ((HOLD || c == 0) && !(alive = warp_wait(&B.afull[HOLD ? c : kChunks - 1], i & 1, err))) break;
       fence_after();
       if (leader) {
 #pragma unroll
@@ -340,12 +375,43 @@ __device__ __forceinline__ void issue_mmas(char* sm, Bars& B, uint32_t tmem, uin
   __syncwarp();
 }
 
+// A ReLU decision of the recompute can differ from the FP32 MLP's where the pre-activation is within
+// their errors of zero, and one flipped mask moves that sample's whole gradient through the unit.  Unit n
+// of layer 1 is uncertain when |z1_n| <= eps ||W1_n|| ||x||, unit n of layer 2 when |z2_n| <= eps ||W2_n||
+// (||h1|| + ||x|| ||W1||_F) (its own sum plus layer 1's errors carried through W2); samples with an
+// uncertain unit are listed (their sorted index, in rec_key; count in hdr[4]) and taken again by k_fwd_fix.
+// With three parts the dropped products are ~2^-24 of a term; what is left is rounding: the tensor core's
+// ~8 truncations at full size and the FP32 chain's ~K roundings, each some 2^-24 of ||w o x|| ~ ||w||
+// ||x|| / sqrt(K), a total of ~2^-24 ||w|| ||x||: eps = 2^-21 leaves a factor of 8.  0.5% of the samples
+// of the 8192-ray workload are listed (8.6% with two parts and 2^-17).
+constexpr float kEps = 4.76837158203125e-07f;  // 2^-21
+
+// What is written besides (c, w): nothing (a render), the ReLU masks (a backward follows), or the masks
+// and the weight gradients' operands x, h1 and h2 (WgStage: the first two BF16 parts).
+enum class Out { Colour, Masks, Stage };
+
+// row group g (8 rows) of the staged operand at offset op (R rows) of one sample, whose rows start at col
+__device__ __forceinline__ void stage_put(char* col, int op, int R, int g, const uint4& hi, const uint4& lo) {
+  *reinterpret_cast<uint4*>(col + op + 256 * g) = hi;
+  *reinterpret_cast<uint4*>(col + op + 32 * R + 256 * g) = lo;
+}
+// HOLD: E1 takes all of its 64 accumulator columns into registers before it converts them, so that layer 2
+// can overwrite them as soon as the first chunk of h1 is written.  Without it E1 (and E2) load 32 at a
+// time, layer 2 waits for both chunks, and G has the registers for more loads in flight.
+// A render holds (62.5 M samples, NP = 3: 8.7 ms against 10.1); a recompute, whose E1 and E2 also keep
+// masks, norms and staging addresses, does not (2.06 M samples of an FP32 grid: 0.51 ms against 0.59,
+// with the staging 0.74 against 0.96 on 1.8 M: the held columns spilled).
+template <Out OUT>
+__host__ __device__ constexpr bool hold() { return OUT == Out::Colour; }
+
 // CC, NF: channels and frequencies as constants (12 and 4), or 0: known at run time only.
-template <int NP, int CC, int NF>
+template <int NP, int CC, int NF, Out OUT>
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs mlp, RenderWs w, const void* feat_,
                                                            int f16) {
   using namespace tc;
   using S = Smem<NP>;
+  constexpr bool HOLD = hold<OUT>();
+  using RG = Regs<HOLD>;
   extern __shared__ __align__(1024) char sm[];
   Bars& B = *(Bars*)(sm + S::bars);
   uint32_t* err = &w.hdr[0];
@@ -365,12 +431,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
     p[6] = mlp.w3[2 * kHidden + i];
   }
   if (threadIdx.x < 4) b3s[threadIdx.x] = threadIdx.x < 3 ? mlp.b3[threadIdx.x] : 0.0f;
+  float* nrm = (float*)(sm + S::nrm);
+  if constexpr (OUT != Out::Colour) {  // a warp per row
+    for (int r = wid; r < 2 * kHidden; r += kThreads / 32) {
+      const int in = r < kHidden ? mlp.in_dim : kHidden;
+      const float* row = r < kHidden ? mlp.w1 + r * in : mlp.w2 + (r - kHidden) * in;
+      float q = 0.0f;
+      for (int k = lane; k < in; k += 32) q = fmaf(row[k], row[k], q);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      if (lane == 0) nrm[r] = sqrtf(q);
+    }
+  }
   if (threadIdx.x == 0) {
     for (int b = 0; b < 2; b++) {
       mbar_init(&B.xfull[b], kGatWarps);
       mbar_init(&B.l1done[b], 1);
       mbar_init(&B.l2done[b], 1);
       mbar_init(&B.dfree[b], kEpiWarps);
+      mbar_init(&B.hfull[b], kEpiWarps);
     }
     for (int c = 0; c < kChunks; c++) {
       mbar_init(&B.afull[c], kEpiWarps);
@@ -391,6 +470,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
   fence_before();
   __syncthreads();
   fence_after();
+  if constexpr (OUT != Out::Colour) {
+    if (wid == 0) {
+      float q = 0.0f;
+      for (int k = lane; k < kHidden; k += 32) q = fmaf(nrm[k], nrm[k], q);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      if (lane == 0) nrm[2 * kHidden] = sqrtf(q);
+    }
+    __syncthreads();
+  }
   const uint32_t tmem = B.tmem;
   const uint32_t dcol = tmem + Tmem<NP>::acc;  // accumulator of tile i: dcol + 128 (i & 1)
 
@@ -400,17 +489,34 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
 
   if (wid < kE2) {
     // ------------------------------------------------------------------ E1: layer 1 -> h1
-    regs_up<kRegsE1>();
-    const int h = wid >> 2;
+    set_regs<RG::e1>();
+    const int h = wid >> 2, m = (wid & 3) * 32 + lane;
     const uint32_t lanes = (uint32_t)((wid & 3) * 32) << 16;
+    const float4* meta = (const float4*)(sm + S::meta);
+    (void)m;
+    (void)meta;
     bool alive = true;
     for (uint32_t i = 0; i < n && alive; i++) {
       if (!(alive = warp_wait(&B.l1done[i & 1], (i >> 1) & 1, err))) break;
+      uint32_t rid = 0xffffffffu, mw[2] = {0u, 0u}, unsure = 0u;
+      float2 hh = make_float2(0.f, 0.f);  // ||h1||^2 of this half
+      float tx = 0.0f;
+      char* stg = nullptr;
+      if constexpr (OUT != Out::Colour) {
+        if (!(alive = warp_wait(&B.mfull[i % kMeta], (i / kMeta) & 1, err))) break;
+        const float4 md = meta[(i % kMeta) * kTile + m];
+        rid = __float_as_uint(md.x);
+        tx = -kEps * sqrtf(md.w);
+        if (OUT == Out::Stage) stg = w.stage + stage_col(__float_as_uint(md.z));
+      }
       fence_after();
-      float v[64];
-      load_half(dcol + 128u * (i & 1) + lanes, h, v);  // all of it: layer 2 overwrites these columns
+      float v[HOLD ? 64 : 32];
+      if constexpr (HOLD) load_half(dcol + 128u * (i & 1) + lanes, h, v);
 #pragma unroll
       for (int q4 = 0; q4 < 4; q4++) {  // 16 units at a time, 4 / kChunks of them per chunk
+        if constexpr (!HOLD) {
+          if (q4 % 2 == 0) load_quarter(dcol + 128u * (i & 1) + lanes, h, q4 / 2, v);
+        }
         constexpr int kPer = 4 / kChunks;
         const int c = q4 / kPer;
         const float4* b4 = reinterpret_cast<const float4*>(b1s + 32 * q4 + 16 * h);
@@ -418,17 +524,36 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
 #pragma unroll
         for (int q = 0; q < 4; q++) {
           const float4 b = b4[q];
-          const float* z = v + 16 * q4 + 4 * q;
+          const float* z = v + 16 * (HOLD ? q4 : q4 % 2) + 4 * q;
           const float2 u0 = add2(make_float2(z[0], z[1]), make_float2(b.x, b.y));
           const float2 u1 = add2(make_float2(z[2], z[3]), make_float2(b.z, b.w));
+          const float2 r0 = make_float2(fmaxf(u0.x, 0.0f), fmaxf(u0.y, 0.0f));
+          const float2 r1 = make_float2(fmaxf(u1.x, 0.0f), fmaxf(u1.y, 0.0f));
+          if constexpr (OUT != Out::Colour) {
+            mw[q4 & 1] |= ((u0.x > 0.0f ? 1u : 0u) | (u0.y > 0.0f ? 2u : 0u) | (u1.x > 0.0f ? 4u : 0u) |
+                           (u1.y > 0.0f ? 8u : 0u)) << (8 * q + 4 * (q4 >> 1));
+            const float4 nw = reinterpret_cast<const float4*>(nrm + 32 * q4 + 16 * h)[q];
+            // (the sign of |z| - eps ||W_n|| ||x||: set where uncertain; a NaN decides like the FP32 MLP)
+            unsure |= __float_as_uint(fmaf(tx, nw.x, fabsf(u0.x))) | __float_as_uint(fmaf(tx, nw.y, fabsf(u0.y)));
+            unsure |= __float_as_uint(fmaf(tx, nw.z, fabsf(u1.x))) | __float_as_uint(fmaf(tx, nw.w, fabsf(u1.y)));
+            hh = fma2(r0, r0, hh);
+            hh = fma2(r1, r1, hh);
+          }
           uint32_t p0[NP], p1[NP];
-          split2<NP>(make_float2(fmaxf(u0.x, 0.0f), fmaxf(u0.y, 0.0f)), p0);
-          split2<NP>(make_float2(fmaxf(u1.x, 0.0f), fmaxf(u1.y, 0.0f)), p1);
+          split2<NP>(r0, p0);
+          split2<NP>(r1, p1);
 #pragma unroll
           for (int k = 0; k < NP; k++) {
             o[k][2 * q] = p0[k];
             o[k][2 * q + 1] = p1[k];
           }
+        }
+        if (OUT == Out::Stage && rid != 0xffffffffu) {
+#pragma unroll
+          for (int u = 0; u < 2; u++)
+            stage_put(stg, WgStage::h1, kHidden, 4 * q4 + 2 * h + u,
+                      make_uint4(o[0][4 * u], o[0][4 * u + 1], o[0][4 * u + 2], o[0][4 * u + 3]),
+                      make_uint4(o[1][4 * u], o[1][4 * u + 1], o[1][4 * u + 2], o[1][4 * u + 3]));
         }
         // the hi part's other buffer is free (layer 2 of tile i - 2 was issued before layer 1 of tile i)
         tmem_st8(tmem + lanes + h1_col(0, i) + 16u * q4 + 8u * h, o[0]);
@@ -444,10 +569,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
           warp_arrive(&B.afull[c]);
         }
       }
+      if constexpr (OUT != Out::Colour) {
+        if (!alive) break;
+        ((float*)(sm + S::hs))[((i & 1) * 2 + h) * kTile + m] =
+            __uint_as_float(__float_as_uint(hh.x + hh.y) | (unsure & 0x80000000u));
+        warp_arrive(&B.hfull[i & 1]);
+        if (rid != 0xffffffffu)
+          *reinterpret_cast<uint2*>(reinterpret_cast<char*>(w.rec_mask + 2 * (size_t)rid) + 8 * h) =
+              make_uint2(mw[0], mw[1]);
+      }
     }
   } else if (wid < kG) {
     // ------------------------------------------------------------------ E2: layer 2 -> layer 3 -> record
-    regs_up<kRegsE2>();
+    set_regs<RG::e2>();
     const int h = (wid - kE2) >> 2, m = (wid & 3) * 32 + lane;
     const uint32_t lanes = (uint32_t)((wid & 3) * 32) << 16;
     float4* zbuf = (float4*)(sm + S::z);
@@ -457,30 +591,78 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
       if (!warp_wait(&B.mfull[t % kMeta], (t / kMeta) & 1, err)) break;
       fence_after();
       const float4 md = meta[(t % kMeta) * kTile + m];
-      float v[64];
-      load_half(dcol + 128u * (t & 1) + lanes, h, v);  // all of it, to free the accumulator at once
-      fence_before();
-      warp_arrive(&B.dfree[t & 1]);
+      const uint32_t rid = __float_as_uint(md.x);
+      uint32_t mw[2] = {0u, 0u}, sh[2][4], unsure = 0u;
+      float th = 0.0f;
+      if constexpr (OUT != Out::Colour) {
+        if (!warp_wait(&B.hfull[t & 1], (t >> 1) & 1, err)) break;
+        const float* hs = (const float*)(sm + S::hs) + (t & 1) * 2 * kTile + m;
+        unsure = __float_as_uint(hs[0]) | __float_as_uint(hs[kTile]);
+        th = -kEps * (sqrtf(fabsf(hs[0]) + fabsf(hs[kTile])) + sqrtf(md.w) * nrm[2 * kHidden]);
+      }
+      char* stg = OUT == Out::Stage ? w.stage + stage_col(__float_as_uint(md.z)) : nullptr;
+      (void)mw;
+      (void)sh;
+      (void)stg;
+      (void)th;
+      float v[HOLD ? 64 : 32];
+      if constexpr (HOLD) {  // all of it, to free the accumulator at once
+        load_half(dcol + 128u * (t & 1) + lanes, h, v);
+        fence_before();
+        warp_arrive(&B.dfree[t & 1]);
+      }
       float2 z0 = make_float2(0.f, 0.f), z1 = z0, z2 = z0;
       const float4* l4 = reinterpret_cast<const float4*>(l3) + 16 * h;  // two per pair of units
 #pragma unroll
       for (int q = 0; q < 32; q++) {
+        if constexpr (!HOLD) {
+          if (q % 16 == 0) load_quarter(dcol + 128u * (t & 1) + lanes, h, q / 16, v);
+          if (q == 16) {
+            fence_before();
+            warp_arrive(&B.dfree[t & 1]);
+          }
+        }
         const float4 a = l4[32 * (q / 8) + 2 * (q % 8)], b = l4[32 * (q / 8) + 2 * (q % 8) + 1];
-        float2 u = add2(make_float2(v[2 * q], v[2 * q + 1]), make_float2(a.x, a.y));
+        float2 u = add2(make_float2(v[2 * (HOLD ? q : q % 16)], v[2 * (HOLD ? q : q % 16) + 1]), make_float2(a.x, a.y));
+        if constexpr (OUT != Out::Colour) {
+          mw[(q >> 3) & 1] |= ((u.x > 0.0f ? 1u : 0u) | (u.y > 0.0f ? 2u : 0u)) <<
+                              (8 * ((q & 7) >> 1) + 2 * (q & 1) + 4 * (q >> 4));
+          const float2 nw = *reinterpret_cast<const float2*>(nrm + kHidden + 32 * (q / 8) + 16 * h + 2 * (q % 8));
+          unsure |= __float_as_uint(fmaf(th, nw.x, fabsf(u.x))) | __float_as_uint(fmaf(th, nw.y, fabsf(u.y)));
+        }
         u.x = fmaxf(u.x, 0.0f);
         u.y = fmaxf(u.y, 0.0f);
         z0 = fma2(make_float2(a.z, a.w), u, z0);
         z1 = fma2(make_float2(b.x, b.y), u, z1);
         z2 = fma2(make_float2(b.z, b.w), u, z2);
+        if constexpr (OUT == Out::Stage) {
+          uint32_t p[2];
+          split2<2>(u, p);
+          sh[0][q & 3] = p[0];
+          sh[1][q & 3] = p[1];
+          if ((q & 3) == 3 && rid != 0xffffffffu)  // 8 units complete
+            stage_put(stg, WgStage::h2, kHidden, 4 * (q >> 3) + 2 * h + ((q >> 2) & 1),
+                      make_uint4(sh[0][0], sh[0][1], sh[0][2], sh[0][3]), make_uint4(sh[1][0], sh[1][1], sh[1][2], sh[1][3]));
+        }
       }
+      if (OUT != Out::Colour && rid != 0xffffffffu)
+        *reinterpret_cast<uint2*>(reinterpret_cast<char*>(w.rec_mask + 2 * (size_t)rid + 1) + 8 * h) =
+            make_uint2(mw[0], mw[1]);
       float4* zp = &zbuf[(t % kMeta) * kTile + m];
       if (h) {
-        *zp = make_float4(z0.x + z0.y, z1.x + z1.y, z2.x + z2.y, 0.0f);
+        *zp = make_float4(z0.x + z0.y, z1.x + z1.y, z2.x + z2.y, __uint_as_float(unsure));
         warp_arrive(&B.zfull[t % kMeta]);
       } else {
         if (!warp_wait(&B.zfull[t % kMeta], (t / kMeta) & 1, err)) break;
         const float4 o = *zp;
-        const uint32_t rid = __float_as_uint(md.x);
+        if constexpr (OUT != Out::Colour) {  // list the uncertain samples (one atomic per warp)
+          const bool fix = rid != 0xffffffffu && ((unsure | __float_as_uint(o.w)) >> 31);
+          const uint32_t bal = __ballot_sync(0xffffffffu, fix);
+          uint32_t base = 0;
+          if (lane == 0 && bal) base = atomicAdd(&w.hdr[4], (uint32_t)__popc(bal));
+          base = __shfl_sync(0xffffffffu, base, 0);
+          if (fix) w.rec_key[base + __popc(bal & ((1u << lane) - 1u))] = __float_as_uint(md.z);
+        }
         if (rid != 0xffffffffu)
           w.rec_c[rid] = make_float4(sigmoid_f(z0.x + z0.y + o.x + b3s[0]), sigmoid_f(z1.x + z1.y + o.y + b3s[1]),
                                      sigmoid_f(z2.x + z2.y + o.z + b3s[2]), md.y);
@@ -488,6 +670,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
     }
   } else if (wid < kM) {
     // ------------------------------------------------------------------ G: the input rows
+    set_regs<RG::g>();
     const int m = (wid & 3) * 32 + lane;
     const uint32_t grp = (uint32_t)(wid - kG) / kGatWarps;  // takes tiles grp, grp + 2, ...
     const int C = CC ? CC : g.C, n_freq = NF ? NF : mlp.n_freq, Br = g.brick;
@@ -516,6 +699,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
         d[2] = qd.w;
         md.x = qd.x;
         md.y = pw.w;
+        md.z = __uint_as_float(td.x + m);  // its place in the sorted order
         const int bx = (int)(td.w & 0xFFFFu), by = (int)(td.w >> 16), bz = (int)((td.y >> 8) & 0x1FFFu);
         int i0[3];
         float f[3];
@@ -530,6 +714,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
       }
       if (i + 2 < n) fetch(i + 2);
       if (CC && NF && valid) encode<NF>(d, x + CC);
+      if constexpr (OUT != Out::Colour) {  // ||x||^2 (the encoding's part below, if it is not in x yet)
+#pragma unroll
+        for (int k = 0; k < kK1; k++) md.w = fmaf(x[k], x[k], md.w);
+      }
       // x's buffer: layer 1 of tile i - 2 has read it
       if (i >= 2 && !warp_wait(&B.l1done[i & 1], ((i >> 1) - 1) & 1, err)) break;
       char* xb = sm + S::x + (int)(i & 1) * NP * kXBytes;
@@ -539,6 +727,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
         split_row<NP>(x + k0, q);
 #pragma unroll
         for (int p = 0; p < NP; p++) *reinterpret_cast<uint4*>(xb + p * kXBytes + kmaj_off(m, k0, kK1)) = q[p];
+        if (OUT == Out::Stage && CC && NF && valid)
+          stage_put(w.stage + stage_col(__float_as_uint(md.z)), WgStage::x, kMaxIn, k0 / 8, q[0], q[1]);
       }
       if (!(CC && NF) && valid) {
         // channels known at run time only: the encoding is written over columns C .. element by element
@@ -554,6 +744,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
 #pragma unroll
           for (int u = 0; u < 2; u++) {
             const int k = C + j + u;
+            if (OUT != Out::Colour && j + u < ne) md.w = fmaf(e[j + u], e[j + u], md.w);
             if (j + u < ne)
 #pragma unroll
               for (int a = 0; a < NP; a++)
@@ -561,6 +752,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
                     (uint16_t)(p[a] >> (16 * u));
           }
         }
+      }
+      if (OUT == Out::Stage && !(CC && NF) && valid) {  // the row as it now stands in shared memory
+#pragma unroll
+        for (int k0 = 0; k0 < kK1; k0 += 8)
+          stage_put(w.stage + stage_col(__float_as_uint(md.z)), WgStage::x, kMaxIn, k0 / 8,
+                    *reinterpret_cast<uint4*>(xb + kmaj_off(m, k0, kK1)),
+                    *reinterpret_cast<uint4*>(xb + kXBytes + kmaj_off(m, k0, kK1)));
       }
       meta[(i % kMeta) * kTile + m] = md;
       fence_proxy_async();
@@ -572,8 +770,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
     }
   } else {
     // ------------------------------------------------------------------ M: the MMAs
-    regs_down<kRegsM>();
-    if (wid == kM && n) issue_mmas<NP>(sm, B, tmem, n, err);
+    set_regs<RG::m>();
+    if (wid == kM && n) issue_mmas<NP, HOLD>(sm, B, tmem, n, err);
   }
   fence_before();
   __syncthreads();
@@ -582,29 +780,41 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
 }
-template <int NP, int CC, int NF>
+template <int NP, int CC, int NF, Out OUT>
 static cicero_status launch(const cicero_grid* grid, const GridGeo& geo, const MlpPtrs& mlp, const RenderWs& ws,
                             cudaStream_t st) {
-  auto kern = k_mlp_split<NP, CC, NF>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<NP>::bytes);
+  auto kern = k_mlp_split<NP, CC, NF, OUT>;
+  constexpr int smem = OUT == Out::Colour ? Smem<NP>::bytes : Smem<NP>::bytes_bwd;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_mlp_split)");
   {
     ProfScope ps(kStGatherMlp, st);
-    kern<<<num_sms(), kThreads, Smem<NP>::bytes, st>>>(geo, mlp, ws, grid->features, grid->dtype == CICERO_F16);
+    kern<<<num_sms(), kThreads, smem, st>>>(geo, mlp, ws, grid->features, grid->dtype == CICERO_F16);
   }
   count_launches(1);
   e = cudaGetLastError();
   return e == cudaSuccess ? CICERO_OK : cuda_fail(e, "k_mlp_split");
 }
 
+template <int NP, Out OUT>
+static cicero_status launch_channels(const cicero_grid* grid, const GridGeo& geo, const MlpPtrs& mlp,
+                                     const RenderWs& ws, cudaStream_t st) {
+  return geo.C == 12 && mlp.n_freq == 4 ? launch<NP, 12, 4, OUT>(grid, geo, mlp, ws, st)
+                                        : launch<NP, 0, 0, OUT>(grid, geo, mlp, ws, st);
+}
+
 }  // namespace ms
 
 cicero_status launch_mlp_split(const cicero_grid* grid, const GridGeo& geo, int parts, const MlpPtrs& mlp,
                                const RenderWs& ws, cudaStream_t st) {
-  const bool c12 = geo.C == 12 && mlp.n_freq == 4;
-  if (parts == 3)
-    return c12 ? ms::launch<3, 12, 4>(grid, geo, mlp, ws, st) : ms::launch<3, 0, 0>(grid, geo, mlp, ws, st);
-  return c12 ? ms::launch<2, 12, 4>(grid, geo, mlp, ws, st) : ms::launch<2, 0, 0>(grid, geo, mlp, ws, st);
+  return parts == 3 ? ms::launch_channels<3, ms::Out::Colour>(grid, geo, mlp, ws, st)
+                    : ms::launch_channels<2, ms::Out::Colour>(grid, geo, mlp, ws, st);
+}
+
+cicero_status launch_mlp_recompute(const cicero_grid* grid, const GridGeo& geo, const MlpPtrs& mlp, const RenderWs& ws,
+                                   cudaStream_t st) {
+  return ws.stage ? ms::launch_channels<3, ms::Out::Stage>(grid, geo, mlp, ws, st)
+                  : ms::launch_channels<3, ms::Out::Masks>(grid, geo, mlp, ws, st);
 }
 
 }  // namespace cicero

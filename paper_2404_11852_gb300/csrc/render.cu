@@ -851,7 +851,7 @@ __global__ void __launch_bounds__(256, 4) k_scatter(RaySrc src, RenderWs w) {
 }
 
 // -------------------------------------------------------------------------------------------
-// FP32 SIMT MLP over 128-sample tiles: the backward's fix-up of uncertain samples and cicero_mlp_eval.
+// FP32 SIMT MLP over 128-sample tiles (cicero_mlp_eval).
 
 constexpr int kK1 = kMaxIn;  // padded input width of layer 1
 
@@ -866,7 +866,6 @@ struct F32Smem {
   static constexpr int x = b3 + 16;                              // [48][128] inputs
   static constexpr int h = x + kK1 * kTile * 4;                  // [128][128]
   static constexpr int end = ((h + kHidden * kTile * 4 + 127) / 128) * 128;
-  static constexpr int masks = end;                              // the fix-up's ReLU bytes [2][16][128]
 };
 
 // acc[i][j]: rows {tm*4+i, 64+tm*4+(i-4)}, cols {tn*4+j, 64+tn*4+(j-4)}; A, B k-major [K][128].
@@ -950,22 +949,7 @@ __device__ __forceinline__ void nbar_sync(int id, int n) { asm volatile("bar.syn
 // Three-layer MLP of the 128 samples whose inputs are in X [48][128] (rows in_dim.. zero);
 // threads < 128 return c of sample m = threadIdx.x.  Run by the 256 MLP threads (threadIdx.x < 256), which synchronise on
 // their own named barrier.
-// This thread's ReLU bits of one layer into msk [16][128] bytes: byte (tn, m) holds units
-// tn * 4 + j (bit j) and 64 + tn * 4 + j (bit 4 + j) of sample m, as relu(acc + bias) > 0 decides.
-__device__ __forceinline__ void store_relu_bits(const float acc[8][8], const float* bias, uint8_t* msk, int tm,
-                                                int tn) {
-#pragma unroll
-  for (int i = 0; i < 8; i++) {
-    uint32_t byte = 0;
-#pragma unroll
-    for (int j = 0; j < 8; j++) byte |= (acc[i][j] + bias[gemm_row(tn, j)] > 0.f ? 1u : 0u) << j;
-    msk[tn * kTile + gemm_row(tm, i)] = (uint8_t)byte;
-  }
-}
-
-// msk (may be NULL): [2][16][128] bytes receiving the ReLU masks of layers 1 and 2 (store_relu_bits).
-__device__ __forceinline__ void mlp_f32_tile(char* sm, const float* X, float c[3], int in_dim,
-                                             uint8_t* msk = nullptr) {
+__device__ __forceinline__ void mlp_f32_tile(char* sm, const float* X, float c[3], int in_dim) {
   const float* w1t = (const float*)(sm + F32Smem::w1t);
   const float* w2t = (const float*)(sm + F32Smem::w2t);
   const float* w3 = (const float*)(sm + F32Smem::w3);
@@ -980,7 +964,6 @@ __device__ __forceinline__ void mlp_f32_tile(char* sm, const float* X, float c[3
 #pragma unroll
     for (int j = 0; j < 8; j++) acc[i][j] = 0.0f;
   simt_gemm(X, w1t, (in_dim + 3) & ~3, tm, tn, acc);  // rows in_dim.. of X and W1^T are zero
-  if (msk) store_relu_bits(acc, b1, msk, tm, tn);
   simt_epilogue(acc, b1, H, tm, tn);
   nbar_sync(kBarMlp, kMlpThreads);
 #pragma unroll
@@ -988,7 +971,6 @@ __device__ __forceinline__ void mlp_f32_tile(char* sm, const float* X, float c[3
 #pragma unroll
     for (int j = 0; j < 8; j++) acc[i][j] = 0.0f;
   simt_gemm(H, w2t, kHidden, tm, tn, acc);
-  if (msk) store_relu_bits(acc, b2, msk + 16 * kTile, tm, tn);
   // layer-2 epilogue fused with layer 3: h2 = relu(acc + b2) stays in registers; this thread's 8
   // hidden units give partial sums z[i][o] = sum_j w3[o][n_j] h2[i][j] for its 8 samples, and the
   // 16 threads that share the samples add theirs through shared memory (P [16][3][128], over H)
@@ -1031,82 +1013,168 @@ __device__ __forceinline__ void mlp_f32_tile(char* sm, const float* X, float c[3
   }
 }
 
-// The samples that the backward's tensor-core forward recompute (k_fwd_x3) listed (a ReLU
-// pre-activation within its error estimate of zero for the split-BF16 products), recomputed with the FP32
-// MLP (mlp_f32_tile): (c, w) and both ReLU masks overwritten.  The list holds sorted record indices
-// (rec_key, count in hdr[4]); 128 samples per step, features interpolated from global memory.
-// Launched only after k_fwd_x3, so C <= 16.
+// The samples that the backward's tensor-core forward recompute (k_mlp_split) listed (a ReLU
+// pre-activation within its error estimate of zero), recomputed with an FP32 MLP: (c, w) and both ReLU
+// masks overwritten.  The list holds sorted record indices (rec_key, count in hdr[4]).
+// A warp takes four samples, a lane four hidden units of each: every unit's sum runs over its inputs in
+// order, one FMA each, as in mlp_f32_tile, whose decisions these are.  A few samples in a thousand are
+// listed, so what counts is the time of a short list: 128-sample tiles of a block took 50 us for 170 K
+// samples of which ~900 are listed.
+constexpr int kFixS = 4;                    // samples per warp
+struct FixSmem {
+  static constexpr int LD = kHidden + 4;    // row stride of the transposed weights: conflict-free both ways
+  static constexpr int w1t = 0;                              // [48][LD]
+  static constexpr int w2t = w1t + kK1 * LD * 4;             // [128][LD]
+  static constexpr int prm = w2t + kHidden * LD * 4;         // b1 [128], b2 [128], w3 [3][128], b3 [4]
+  static constexpr int xh = prm + (5 * kHidden + 4) * 4;     // per warp: inputs [48][4], then h1 [128][4]
+  static constexpr int warp_bytes = (kK1 + kHidden) * kFixS * 4;
+  static constexpr int bytes = xh + 8 * warp_bytes;
+  static_assert(xh % 16 == 0 && w2t % 16 == 0, "alignment");
+};
+
+// W [128][K] (row-major, global) transposed into dst [K][LD], 4 rows x 8 columns per warp and step
+__device__ __forceinline__ void load_transposed(float* dst, const float* w, int K) {
+  const int lane = threadIdx.x & 31, kb = (K + 7) / 8, n_blk = (kHidden / 4) * kb;
+#pragma unroll 16
+  for (int i = threadIdx.x >> 5; i < n_blk; i += 8) {
+    const int n = (i / kb) * 4 + (lane >> 3), k = (i % kb) * 8 + (lane & 7);
+    if (k < K) dst[k * FixSmem::LD + n] = __ldg(w + n * K + k);
+  }
+}
+
+// acc[u][s] = sum_k in[k][s] wt[k][4 lane + u], k ascending
+__device__ __forceinline__ void fix_layer(const float* wt, const float4* in, int K, float acc[4][kFixS]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int u = 0; u < 4; u++)
+#pragma unroll
+    for (int s = 0; s < kFixS; s++) acc[u][s] = 0.0f;
+#pragma unroll 4
+  for (int k = 0; k < K; k++) {
+    const float4 a = in[k], b = *reinterpret_cast<const float4*>(wt + k * FixSmem::LD + 4 * lane);
+    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int u = 0; u < 4; u++)
+#pragma unroll
+      for (int s = 0; s < kFixS; s++) acc[u][s] = fmaf(av[s], bv[u], acc[u][s]);
+  }
+}
+
 template <typename T>
-__global__ void __launch_bounds__(kMlpThreads, 1) k_fwd_fix(GridGeo g, MlpPtrs mlp, RenderWs w,
-                                                           const T* __restrict__ feat) {
+__global__ void __launch_bounds__(256, 1) k_fwd_fix(GridGeo g, MlpPtrs mlp, RenderWs w, const T* __restrict__ feat) {
   extern __shared__ __align__(128) char sm[];
-  float* X = (float*)(sm + F32Smem::x);
-  uint8_t* msk = (uint8_t*)(sm + F32Smem::masks);  // [2][16][128] ReLU bytes (store_relu_bits)
-  load_mlp_f32_smem(sm, mlp);
   const uint32_t n = w.hdr[4];
-  const int C = g.C, m = threadIdx.x;
-  const int ne = 3 + 6 * mlp.n_freq;
-  const int ms = m & (kTile - 1);  // the step's sample of this thread: threads < 128 interpolate its
-                                   // features, the others encode its direction, side by side
-  for (uint32_t base = blockIdx.x * kTile; base < n; base += gridDim.x * kTile) {
-    const bool valid = m < kTile && base + m < n;
-    const bool has = base + ms < n;
-    uint32_t si = 0;
-    __syncthreads();  // the weights, or the previous step's reads of X and the masks
-    if (has) si = w.rec_key[base + ms];
-    if (m < kTile) {
-      float fx[16];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t n_grp = (n + kFixS - 1) / kFixS;
+  if (blockIdx.x >= n_grp) return;  // no group for this block: the weights are not needed
+  float* w1t = (float*)(sm + FixSmem::w1t);
+  float* w2t = (float*)(sm + FixSmem::w2t);
+  float* b1 = (float*)(sm + FixSmem::prm);
+  float* b2 = b1 + kHidden;
+  float* w3 = b2 + kHidden;
+  float* b3 = w3 + 3 * kHidden;
+  load_transposed(w1t, mlp.w1, mlp.in_dim);
+  load_transposed(w2t, mlp.w2, kHidden);
+  for (int i = threadIdx.x; i < 3 * kHidden; i += 256) w3[i] = mlp.w3[i];
+  for (int i = threadIdx.x; i < kHidden; i += 256) {
+    b1[i] = mlp.b1[i];
+    b2[i] = mlp.b2[i];
+  }
+  if (threadIdx.x < 3) b3[threadIdx.x] = mlp.b3[threadIdx.x];
+  __syncthreads();
+  float* X = (float*)(sm + FixSmem::xh + wid * FixSmem::warp_bytes);  // [48][4]
+  float* H = X + kK1 * kFixS;                                          // [128][4]
+  const int C = g.C, sub = lane & 7, sm_i = lane >> 3;  // this lane's sample of the group and its share of it
+  // groups in turn over the blocks, then over their warps: a short list spreads over the SMs
+  for (uint32_t grp = blockIdx.x + wid * gridDim.x; grp < n_grp; grp += 8 * gridDim.x) {
+    const uint32_t at = grp * kFixS + sm_i;
+    const bool has = at < n;
+    const uint32_t si = has ? w.rec_key[at] : 0u;
+    const float4 pw = has ? w.srt[si].pw : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 qd = has ? w.srt[si].qd : make_float4(0.f, 0.f, 0.f, 0.f);
+    // features: lane (sample, sub) takes channels sub and sub + 8, corner by corner
+    float fx[2] = {0.0f, 0.0f};
+    {
+      const float p[3] = {pw.x, pw.y, pw.z};
+      int i0[3];
+      float f[3];
+      if (has && index_sample(g, p, i0, f)) {
 #pragma unroll
-      for (int c = 0; c < 16; c++) fx[c] = 0.0f;
-      if (has) {
-        const float4 pw = w.srt[si].pw;
-        const float p[3] = {pw.x, pw.y, pw.z};
-        int i0[3];
-        float f[3];
-        if (index_sample(g, p, i0, f)) {
+        for (int q = 0; q < 8; q++) {
+          const float wq = ((q & 1) ? f[0] : 1.f - f[0]) * (((q >> 1) & 1) ? f[1] : 1.f - f[1]) *
+                           ((q >> 2) ? f[2] : 1.f - f[2]);
+          const T* v = feat + (((size_t)(i0[2] + (q >> 2)) * g.n[1] + (i0[1] + ((q >> 1) & 1))) * g.n[0] +
+                               (i0[0] + (q & 1))) * C;
 #pragma unroll
-          for (int q = 0; q < 8; q++) {  // corners outer, channels inner: every load in flight at once
-            const float wq = ((q & 1) ? f[0] : 1.f - f[0]) * (((q >> 1) & 1) ? f[1] : 1.f - f[1]) *
-                             ((q >> 2) ? f[2] : 1.f - f[2]);
-            const size_t vx = ((size_t)(i0[2] + (q >> 2)) * g.n[1] + (i0[1] + ((q >> 1) & 1))) * g.n[0] +
-                              (i0[0] + (q & 1));
-            const T* v = feat + vx * C;
-#pragma unroll
-            for (int c = 0; c < 16; c++)
-              if (c < C) fx[c] = fmaf(wq, ldf(v + c), fx[c]);
-          }
+          for (int u = 0; u < 2; u++)
+            if (sub + 8 * u < C) fx[u] = fmaf(wq, ldf(v + sub + 8 * u), fx[u]);
         }
       }
-#pragma unroll
-      for (int c = 0; c < 16; c++)
-        if (c < C) X[c * kTile + m] = fx[c];
-    } else {
-      float e[3 + 6 * 7];
-      if (has) {
-        const float4 qd = w.srt[si].qd;
-        const float d[3] = {qd.y, qd.z, qd.w};
-        encode_dir(d, mlp.n_freq, e);
-        for (int j = 0; j < ne; j++) X[(C + j) * kTile + ms] = e[j];
-      } else {
-        for (int j = 0; j < ne; j++) X[(C + j) * kTile + ms] = 0.0f;
-      }
-      for (int j = C + ne; j < kK1; j++) X[j * kTile + ms] = 0.0f;
     }
-    __syncthreads();
-    float c[3];
-    mlp_f32_tile(sm, X, c, mlp.in_dim, msk);
-    if (valid) {
-      const uint32_t rid = __float_as_uint(w.srt[si].qd.x);
-      w.rec_c[rid] = make_float4(c[0], c[1], c[2], w.srt[si].pw.w);
-      uint32_t v[8];
+    __syncwarp();  // the previous group's reads of X and H
 #pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const uint8_t* src = msk + (q >> 2) * 16 * kTile + (q & 3) * 4 * kTile + m;
-        v[q] = (uint32_t)src[0] | ((uint32_t)src[kTile] << 8) | ((uint32_t)src[2 * kTile] << 16) |
-               ((uint32_t)src[3 * kTile] << 24);
+    for (int u = 0; u < 2; u++)
+      if (sub + 8 * u < C) X[(sub + 8 * u) * kFixS + sm_i] = fx[u];
+    if (sub < 3) {  // the encoding of one axis (encode_dir)
+      const float d = sub == 0 ? qd.y : (sub == 1 ? qd.z : qd.w);
+      float s, c;
+      sincosf(d, &s, &c);
+      X[(C + sub) * kFixS + sm_i] = d;
+      for (int k = 0; k < mlp.n_freq; k++) {
+        X[(C + 3 + 6 * k + sub) * kFixS + sm_i] = s;
+        X[(C + 6 + 6 * k + sub) * kFixS + sm_i] = c;
+        const float s2 = 2.0f * s * c;
+        c = 1.0f - 2.0f * s * s;
+        s = s2;
       }
-      w.rec_mask[2 * (size_t)rid] = make_uint4(v[0], v[1], v[2], v[3]);
-      w.rec_mask[2 * (size_t)rid + 1] = make_uint4(v[4], v[5], v[6], v[7]);
+    }
+    __syncwarp();
+    float acc[4][kFixS];
+    uint32_t rid[kFixS];
+#pragma unroll
+    for (int s = 0; s < kFixS; s++) rid[s] = __shfl_sync(0xffffffffu, has ? __float_as_uint(qd.x) : 0xffffffffu, 8 * s);
+    // the lane's ReLU bits of layer `layer` -> the samples' mask words (rec_mask layout)
+    auto put_masks = [&](const float* b, int layer) {
+#pragma unroll
+      for (int s = 0; s < kFixS; s++) {
+        uint32_t v = 0;
+#pragma unroll
+        for (int u = 0; u < 4; u++) v |= (acc[u][s] + b[4 * lane + u] > 0.f ? 1u : 0u) << u;
+        v <<= (lane & 3) * 8 + 4 * (lane >> 4);
+        v |= __shfl_xor_sync(0xffffffffu, v, 1);
+        v |= __shfl_xor_sync(0xffffffffu, v, 2);
+        v |= __shfl_xor_sync(0xffffffffu, v, 16);
+        const int word = lane >> 2;  // of lanes 0, 4, 8, 12
+        if ((lane & 19) == 0 && rid[s] != 0xffffffffu)
+          reinterpret_cast<uint32_t*>(w.rec_mask + 2 * (size_t)rid[s] + layer)[((word & 1) << 1) | (word >> 1)] = v;
+      }
+    };
+    fix_layer(w1t, reinterpret_cast<const float4*>(X), mlp.in_dim, acc);
+    put_masks(b1, 0);
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const float bu = b1[4 * lane + u];
+      *reinterpret_cast<float4*>(H + (4 * lane + u) * kFixS) =
+          make_float4(fmaxf(acc[u][0] + bu, 0.f), fmaxf(acc[u][1] + bu, 0.f), fmaxf(acc[u][2] + bu, 0.f),
+                      fmaxf(acc[u][3] + bu, 0.f));
+    }
+    __syncwarp();
+    fix_layer(w2t, reinterpret_cast<const float4*>(H), kHidden, acc);
+    put_masks(b2, 1);
+#pragma unroll
+    for (int s = 0; s < kFixS; s++) {
+      float z[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        const float h = fmaxf(acc[u][s] + b2[4 * lane + u], 0.f);
+#pragma unroll
+        for (int o = 0; o < 3; o++) z[o] = fmaf(w3[o * kHidden + 4 * lane + u], h, z[o]);
+      }
+#pragma unroll
+      for (int o = 0; o < 3; o++) z[o] = warp_sum(z[o]);
+      const float wgt = __shfl_sync(0xffffffffu, pw.w, 8 * s);
+      if (lane == 0 && rid[s] != 0xffffffffu)
+        w.rec_c[rid[s]] = make_float4(sigmoid_f(z[0] + b3[0]), sigmoid_f(z[1] + b3[1]), sigmoid_f(z[2] + b3[2]), wgt);
     }
   }
 }
@@ -1114,12 +1182,11 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_fwd_fix(GridGeo g, MlpPtrs m
 template <typename T>
 static cicero_status launch_fwd_fix(const GridGeo& geo, const MlpPtrs& mlp, const RenderWs& ws, const void* feat,
                                     cudaStream_t st) {
-  const int smem = F32Smem::masks + 2 * 16 * kTile;
-  cudaError_t e = cudaFuncSetAttribute(k_fwd_fix<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(k_fwd_fix<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, FixSmem::bytes);
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_fwd_fix)");
   {
     ProfScope ps(kStGatherMlp, st);
-    k_fwd_fix<T><<<num_sms(), kMlpThreads, smem, st>>>(geo, mlp, ws, (const T*)feat);
+    k_fwd_fix<T><<<num_sms(), 256, FixSmem::bytes, st>>>(geo, mlp, ws, (const T*)feat);
   }
   count_launches(1);
   e = cudaGetLastError();
@@ -1347,6 +1414,8 @@ static int blocks_for_warps(long long warps, int per_sm) {
   return (int)blocks;
 }
 
+constexpr int kMaxSplitC = 16;  // channels that a split-BF16 render takes
+
 // The brick sizes an FP32 render takes: those whose box fits in shared memory beside the 183,040 bytes
 // that an FP32 MLP's weights and buffers take.  k_mlp_split stages no brick; the limit is the interface's.
 static bool f32_brick_fits(const BrickBox& box) { return 183040 + ((box.box_bytes + 127) & ~127) <= 227 * 1024; }
@@ -1392,14 +1461,11 @@ cicero_status run_render(const cicero_grid* grid, const MlpPtrs& mlp, const Rend
   if (hash) {
     s = launch_gather_mlp_bf16_hash(geo, mlp, ws, *hash, st);  // features from the hash encoding
   } else if (plan.precision == CICERO_MLP_FP32_SPLIT) {
-    // split-BF16 tensor-core MLP, features read from global memory (no staged brick)
-    if (!fwd_x3_supported(geo, mlp))
-      return fail(CICERO_ERR_UNSUPPORTED, "the split-BF16 MLP takes at most 16 feature channels");
+    if (geo.C > kMaxSplitC) return fail(CICERO_ERR_UNSUPPORTED, "the split-BF16 MLP takes at most 16 feature channels");
     s = launch_mlp_split(grid, geo, 2, mlp, ws, st);
-  } else if (ws.rec_mask && fwd_x3_supported(geo, mlp)) {
-    // a backward follows: colours and ReLU masks only, on the tensor cores, then the uncertain
-    // samples again in FP32
-    s = launch_fwd_x3(grid, geo, mlp, ws, st);
+  } else if (ws.rec_mask && tc_backward(geo)) {
+    // a backward follows: colours and ReLU masks, then the uncertain samples again in FP32
+    s = launch_mlp_recompute(grid, geo, mlp, ws, st);
     if (s == CICERO_OK)
       s = f16 ? launch_fwd_fix<__half>(geo, mlp, ws, grid->features, st)
               : launch_fwd_fix<float>(geo, mlp, ws, grid->features, st);

@@ -91,3 +91,31 @@ def test_split_tile_counts(cc, orc, precision, side, n_samples):
         if pix is not None:
             out = {k: v[pix] for k, v in out.items()}
         check_render(out, ref, TOL_SPLIT[precision])
+
+
+@pytest.mark.parametrize("C,dtype,with_mlp", [(4, np.float32, False), (8, np.float16, True), (16, np.float32, True),
+                                              (3, np.float32, True)])
+def test_backward_masks_and_fixup(cc, orc, C, dtype, with_mlp):
+    """The recompute's ReLU masks, its FP32 fix-up and the staged operands at other channel counts: every
+    gradient within 1e-4 relative of the oracle's (a single flipped mask moves d_features by ~1e-3)."""
+    import torch
+    g = scenes.make_grid(32, C, 4, seed=800 + C, dtype=dtype)
+    m = scenes.make_mlp(C, seed=810 + C, random_bias=True)
+    o, d = scenes.random_rays(300, seed=820 + C)
+    sp = scenes.Sampling(near=0.5, far=2.5, n_samples=40, t_stop=0.0)
+    out = orc.render(g, m, sp, rays=(o, d))
+    grad = np.random.default_rng(C).standard_normal((300, 3))
+    grad[out["amb"]] = 0.0
+    want = orc.backward(g, m, sp, grad, rays=(o, d), with_mlp=with_mlp)
+    gd, md, sd = cc.DeviceGrid.from_host(g), cc.DeviceMlp.from_host(m), cc.sampling_from(sp)
+    got = [torch.zeros(g.density.shape, device="cuda"), torch.zeros(g.features.shape, device="cuda"),
+           torch.zeros(m.flat().size, device="cuda") if with_mlp else None]
+    size = cc.cicero_backward_mlp_workspace_size if with_mlp else cc.cicero_backward_workspace_size
+    ws = cc.workspace(size(gd.desc, 300, sd))
+    cc.cicero_render_backward(gd.desc, md.desc, torch.from_numpy(o).cuda(), torch.from_numpy(d).cuda(), sd,
+                              torch.from_numpy(grad.astype(np.float32)).cuda(), *got, ws)
+    cc.cicero_workspace_status(ws)
+    for a, b in zip(got, want):
+        if a is not None:
+            a = a.cpu().double().numpy().ravel()
+            assert np.abs(a - np.ravel(b)).max() <= 1e-4 * np.abs(b).max()
