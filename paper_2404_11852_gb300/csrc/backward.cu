@@ -625,16 +625,29 @@ struct HalfMask {
   }
 };
 
-// A (hi, lo) x B (hi, lo) over K = 16 KSTEPS into the accumulator at d: three products per K step
-template <int KSTEPS = kHidden / 16>
-__device__ __forceinline__ void mma_split(uint32_t d, uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl,
-                                          uint32_t idesc) {
+// A (hi, lo) x B (hi, lo) over K = 128 into the accumulator at d, three products per K step, then the
+// commit to the mbarrier at shared address bar.  Run by a whole warp; one elected lane issues, with
+// operands that are the same for the warp (the instruction reads uniform registers; per-thread
+// descriptors cost some ten instructions per MMA).  Descriptors: their low words.
+template <int N>
+__device__ __forceinline__ void issue_split(uint32_t d, uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl, uint32_t bar) {
+  using namespace tc;
+  constexpr uint32_t hi = desc_hi(kHidden * 16), id = idesc_bf16(N);
+  d = __shfl_sync(0xffffffffu, d, 0);
+  ah = __shfl_sync(0xffffffffu, ah, 0);
+  al = __shfl_sync(0xffffffffu, al, 0);
+  bar = __shfl_sync(0xffffffffu, bar, 0);
+  if (elect_one()) {
+    fence_after();
 #pragma unroll
-  for (int s = 0; s < KSTEPS; s++) {
-    tc::mma_bf16(d, ah + 16u * s, bh + 16u * s, idesc, s > 0 ? 1u : 0u);
-    tc::mma_bf16(d, ah + 16u * s, bl + 16u * s, idesc, 1u);
-    tc::mma_bf16(d, al + 16u * s, bh + 16u * s, idesc, 1u);
+    for (int s = 0; s < kHidden / 16; s++) {
+      mma_u<hi, hi, id>(d, ah + 16u * s, bh + 16u * s, s > 0 ? 1u : 0u);
+      mma_u<hi, hi, id>(d, ah + 16u * s, bl + 16u * s, 1u);
+      mma_u<hi, hi, id>(d, al + 16u * s, bh + 16u * s, 1u);
+    }
+    mma_commit_at(bar);
   }
+  __syncwarp();
 }
 
 // Group grp = tid / 128 takes tiles t_begin + grp, t_begin + grp + 2, ...; thread m = tid mod 128
@@ -687,11 +700,9 @@ __global__ void __launch_bounds__(bt::kThreads, 1) k_bwd_brick_tc(GridGeo g, Mlp
   const uint32_t tmem_base = *tslot;
   const uint32_t tmem = tmem_base + 128u * (uint32_t)grp;                             // this group's columns
   const uint32_t taddr = tmem + ((uint32_t)(((threadIdx.x >> 5) & 3) * 32) << 16);  // this warp's lanes
-  const uint64_t ah = smem_desc(smem_u32(a_hi), 128u, kHidden * 16), al = smem_desc(smem_u32(a_lo), 128u, kHidden * 16);
-  const uint64_t b2h = smem_desc(smem_u32(sm + bt::Smem::w2t_hi), 128u, kHidden * 16);
-  const uint64_t b2l = smem_desc(smem_u32(sm + bt::Smem::w2t_lo), 128u, kHidden * 16);
-  const uint64_t b1h = smem_desc(smem_u32(sm + bt::Smem::w1t_hi), 128u, kHidden * 16);
-  const uint64_t b1l = smem_desc(smem_u32(sm + bt::Smem::w1t_lo), 128u, kHidden * 16);
+  const uint32_t ah = desc_lo(smem_u32(a_hi), 128u), al = desc_lo(smem_u32(a_lo), 128u);
+  const uint32_t b2h = desc_lo(smem_u32(sm + bt::Smem::w2t_hi), 128u), b2l = desc_lo(smem_u32(sm + bt::Smem::w2t_lo), 128u);
+  const uint32_t b1h = desc_lo(smem_u32(sm + bt::Smem::w1t_hi), 128u), b1l = desc_lo(smem_u32(sm + bt::Smem::w1t_lo), 128u);
   uint32_t phase = 0;
   bool alive = true;
 
@@ -785,11 +796,7 @@ __global__ void __launch_bounds__(bt::kThreads, 1) k_bwd_brick_tc(GridGeo g, Mlp
     fence_before();
     group_sync(grp);
     // dh1 = dh2 W2 into the group's columns [0, 128)
-    if (m == 0) {
-      fence_after();
-      mma_split(tmem, ah, al, b2h, b2l, idesc_bf16(kHidden));
-      mma_commit(bar);
-    }
+    if (m < 32) issue_split<kHidden>(tmem, ah, al, b2h, b2l, smem_u32(bar));
     alive = group_sync_and(grp, mbar_wait(bar, phase, &w.hdr[0]));
     fence_after();
     if (!alive) break;
@@ -816,11 +823,7 @@ __global__ void __launch_bounds__(bt::kThreads, 1) k_bwd_brick_tc(GridGeo g, Mlp
     fence_before();
     group_sync(grp);
     // dL/dfeatures = dh1 W1[:, :C] into the group's columns [0, 16)
-    if (m == 0) {
-      fence_after();
-      mma_split(tmem, ah, al, b1h, b1l, idesc_bf16(bt::kN1));
-      mma_commit(bar);
-    }
+    if (m < 32) issue_split<bt::kN1>(tmem, ah, al, b1h, b1l, smem_u32(bar));
     alive = group_sync_and(grp, mbar_wait(bar, phase, &w.hdr[0]));
     fence_after();
     if (!alive) break;
