@@ -48,6 +48,7 @@ __device__ __forceinline__ float warp_sum_b(float v) {
 // B1: per composited sample, (dL/dz3, dL/draw) written over its colour record (rec_c).
 __global__ void __launch_bounds__(256) k_bwd_ray(RaySrc src, Samp s, RenderWs w, const float* __restrict__ d_rgb,
                                                  float act_shift) {
+  dependents_sync();
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -253,6 +254,7 @@ __global__ void __launch_bounds__(256, 1) k_bwd_brick(GridGeo g, RaySrc src, Mlp
     b2[i] = mlp.b2[i];
   }
   __syncthreads();
+  dependents_sync();
 
   const uint32_t n_tiles = w.hdr[1];
   const uint32_t per = (n_tiles + gridDim.x - 1) / gridDim.x;
@@ -705,6 +707,7 @@ __global__ void __launch_bounds__(bt::kThreads, 1) k_bwd_brick_tc(GridGeo g, Mlp
   const uint32_t b1h = desc_lo(smem_u32(sm + bt::Smem::w1t_hi), 128u), b1l = desc_lo(smem_u32(sm + bt::Smem::w1t_lo), 128u);
   uint32_t phase = 0;
   bool alive = true;
+  dependents_sync();
 
   const uint32_t n_tiles = w.hdr[1];
   const uint32_t per = (n_tiles + gridDim.x - 1) / gridDim.x;
@@ -896,6 +899,7 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 // d_mlp once per CTA.  Thread 0 streams the blocks through a ring of kRing buffers with bulk copies
 // (one mbarrier per buffer for the copy, one for the MMAs that read it) and issues the MMAs.
 __global__ void __launch_bounds__(dw::kThreads, 1) k_dw(MlpPtrs mlp, RenderWs w, float* d_mlp) {
+  dependents_sync();
   using namespace tc;
   extern __shared__ __align__(1024) char sm[];
   const int I = mlp.in_dim;
@@ -1068,7 +1072,7 @@ __global__ void __launch_bounds__(dw::kThreads, 1) k_dw(MlpPtrs mlp, RenderWs w,
 cicero_status launch_dw(const MlpPtrs& mlp, const RenderWs& ws, float* d_mlp, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, dw::Smem::bytes);
   if (e == cudaSuccess) {
-    k_dw<<<num_sms(), dw::kThreads, dw::Smem::bytes, st>>>(mlp, ws, d_mlp);
+    launch_kernel(k_dw, num_sms(), dw::kThreads, dw::Smem::bytes, st, mlp, ws, d_mlp);
     e = cudaGetLastError();
   }
   count_launches(1);
@@ -1081,7 +1085,7 @@ static cudaError_t launch_bwd_brick(const RenderPlan& plan, const RaySrc& src, c
                                     int smem, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_bwd_brick<T, WG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  k_bwd_brick<T, WG><<<num_sms(), 256, smem, st>>>(plan.geo, src, mlp, ws, (const T*)feat, d_dens, d_feat, d_mlp);
+  launch_kernel(k_bwd_brick<T, WG>, num_sms(), 256, smem, st, plan.geo, src, mlp, ws, (const T*)feat, d_dens, d_feat, d_mlp);
   return cudaGetLastError();
 }
 
@@ -1099,7 +1103,7 @@ cicero_status run_backward(const cicero_grid* grid, const MlpPtrs& mlp, const Re
   blocks = std::max(1, std::min(blocks, num_sms() * 16));
   {
     ProfScope ps(kStBwdRay, st);
-    k_bwd_ray<<<blocks, 256, 0, st>>>(src, plan.samp, ws, d_rgb, plan.geo.act_shift);
+    launch_kernel(k_bwd_ray, blocks, 256, 0, st, src, plan.samp, ws, d_rgb, plan.geo.act_shift);
   }
   count_launches(2);
   const int smem = BwdSmem::bytes;
@@ -1114,11 +1118,11 @@ cicero_status run_backward(const cicero_grid* grid, const MlpPtrs& mlp, const Re
       if (ws.stage) {
         e = cudaFuncSetAttribute(k_bwd_brick_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_tc);
         if (e == cudaSuccess)
-          k_bwd_brick_tc<true><<<num_sms(), bt::kThreads, smem_tc, st>>>(plan.geo, mlp, ws, d_dens, d_feat);
+          launch_kernel(k_bwd_brick_tc<true>, num_sms(), bt::kThreads, smem_tc, st, plan.geo, mlp, ws, d_dens, d_feat);
       } else {
         e = cudaFuncSetAttribute(k_bwd_brick_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_tc);
         if (e == cudaSuccess)
-          k_bwd_brick_tc<false><<<num_sms(), bt::kThreads, smem_tc, st>>>(plan.geo, mlp, ws, d_dens, d_feat);
+          launch_kernel(k_bwd_brick_tc<false>, num_sms(), bt::kThreads, smem_tc, st, plan.geo, mlp, ws, d_dens, d_feat);
       }
       if (e == cudaSuccess) e = cudaGetLastError();
       if (e != cudaSuccess) return cuda_fail(e, "backward kernels");

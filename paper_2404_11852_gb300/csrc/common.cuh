@@ -329,6 +329,19 @@ __device__ __forceinline__ void encode_dir(const float d[3], int n_freq, float* 
   }
 }
 
+// Programmatic dependent launch: every kernel of a call but the composite is launched while its
+// predecessor on the stream may still run (launch_kernel in internal.h).  A kernel calls
+// dependents_sync() before it touches anything a predecessor wrote or still reads: it waits until the
+// predecessor is complete and its writes visible, and only then lets its own successor start.  So
+// whatever runs before the call (weights into shared memory, barriers, tensor memory) may read what the
+// user passed in: by then every kernel but the immediate predecessor is complete; the first kernel of a
+// call, whose predecessor is the caller's, reads nothing before it.  Data of the predecessor is never
+// read through the read-only path.
+__device__ __forceinline__ void dependents_sync() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 
 __device__ __forceinline__ void set_err(uint32_t* err, uint32_t bits) { atomicOr(err, bits); }

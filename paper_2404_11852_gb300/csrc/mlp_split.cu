@@ -481,6 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
     __syncthreads();
   }
   const uint32_t tmem = B.tmem;
+  dependents_sync();  // the weights are in place by the time the previous kernel has ended
   const uint32_t dcol = tmem + Tmem<NP>::acc;  // accumulator of tile i: dcol + 128 (i & 1)
 
   const uint32_t n_tiles = w.hdr[1];
@@ -789,7 +790,7 @@ static cicero_status launch(const cicero_grid* grid, const GridGeo& geo, const M
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_mlp_split)");
   {
     ProfScope ps(kStGatherMlp, st);
-    kern<<<num_sms(), kThreads, smem, st>>>(geo, mlp, ws, grid->features, grid->dtype == CICERO_F16);
+    launch_kernel(kern, num_sms(), kThreads, smem, st, geo, mlp, ws, grid->features, grid->dtype == CICERO_F16);
   }
   count_launches(1);
   e = cudaGetLastError();

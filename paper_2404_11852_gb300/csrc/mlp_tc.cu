@@ -76,7 +76,19 @@ __device__ __forceinline__ bool gsync_and(int g, bool v) {
   return r != 0;
 }
 
+// 8 consecutive weights
+__device__ __forceinline__ void load8(const float* p, bool vec, float* v) {
+  if (vec) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; j++) v[j] = __ldg(p + j);
+  }
+}
+
 __device__ void load_weights(char* sm, const MlpPtrs& m) {
+#pragma unroll 2
   for (int i = threadIdx.x; i < kHidden * (kK1 / 8); i += blockDim.x) {
     const int n = i / (kK1 / 8), k0 = (i % (kK1 / 8)) * 8;
     float v[8];
@@ -87,13 +99,16 @@ __device__ void load_weights(char* sm, const MlpPtrs& m) {
     }
     store_chunk(sm + Smem::w1, n, k0, kK1, v);
   }
+  const bool vec2 = (reinterpret_cast<uintptr_t>(m.w2) & 15u) == 0;
+#pragma unroll 2
   for (int i = threadIdx.x; i < kHidden * (kK2 / 8); i += blockDim.x) {
     const int n = i / (kK2 / 8), k0 = (i % (kK2 / 8)) * 8;
     float v[8];
+    if (k0 < kHidden) {
+      load8(m.w2 + n * kHidden + k0, vec2, v);
+    } else {
 #pragma unroll
-    for (int j = 0; j < 8; j++) {
-      const int k = k0 + j;
-      v[j] = k < kHidden ? m.w2[n * kHidden + k] : (k == kHidden ? m.b2[n] : 0.0f);  // b2 rides on a 1 column
+      for (int j = 0; j < 8; j++) v[j] = k0 + j == kHidden ? m.b2[n] : 0.0f;  // b2 rides on a 1 column
     }
     store_chunk(sm + Smem::w2, n, k0, kK2, v);
   }
@@ -652,6 +667,7 @@ __global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16(GridGeo g, MlpPtrs m
   extern __shared__ __align__(1024) char sm[];
   Group G = setup(sm, &mlp, groups, box_bytes);
   const uint32_t tmem_base = G.tmem - (uint32_t)(G.g * 128);
+  dependents_sync();  // weights, barriers and tensor memory are set up while the previous kernel ends
   const uint32_t n_tiles = w.hdr[1];
   const uint32_t per = (n_tiles + gridDim.x - 1) / gridDim.x;
   const uint32_t c_begin = blockIdx.x * per, c_end = min(n_tiles, c_begin + per);
@@ -672,6 +688,7 @@ __global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16_hash(GridGeo g, MlpP
   extern __shared__ __align__(1024) char sm[];
   Group G = setup(sm, &mlp, groups, 0);
   const uint32_t tmem_base = G.tmem - (uint32_t)(G.g * 128);
+  dependents_sync();  // weights, barriers and tensor memory are set up while the previous kernel ends
   const uint32_t n_tiles = w.hdr[1];
   const uint32_t per = (n_tiles + gridDim.x - 1) / gridDim.x;
   const uint32_t c_begin = blockIdx.x * per, c_end = min(n_tiles, c_begin + per);
@@ -696,6 +713,7 @@ __global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16_batch(const JobDesc*
   extern __shared__ __align__(1024) char sm[];
   Group G = setup(sm, nullptr, groups, box_bytes);
   const uint32_t tmem_base = G.tmem - (uint32_t)(G.g * 128);
+  dependents_sync();  // weights, barriers and tensor memory are set up while the previous kernel ends
   GridGeo& geo = *(GridGeo*)(sm + Smem::geo);  // the current job's geometry, read by every group
   const MlpPtrs* cur = nullptr;
   int loaded = -1;
@@ -726,6 +744,7 @@ __global__ void __launch_bounds__(512, 1) k_gather_mlp_bf16_batch(const JobDesc*
 __global__ void __launch_bounds__(512, 1) k_mlp_eval_bf16(MlpPtrs mlp, const float* x, int M, float* c, uint32_t* err) {
   using namespace tc;
   extern __shared__ __align__(1024) char sm[];
+  dependents_sync();  // the call's first kernel: the caller's last one may have written the weights
   Group G = setup(sm, &mlp, kMaxGroups, 0);
   const uint32_t tmem_base = G.tmem - (uint32_t)(G.g * 128);
   const int ntile = (M + kTile - 1) / kTile;
@@ -801,7 +820,7 @@ static cicero_status launch_tc(const GridGeo& geo, const MlpPtrs& mlp, const Ren
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_gather_mlp_bf16)");
   {
     ProfScope ps(kStGatherMlp, st);
-    kern<<<num_sms(), 128 * groups, smem, st>>>(geo, mlp, ws, map, (const T*)feat, box.vb, box.vx, box_bytes, groups);
+    launch_kernel(kern, num_sms(), 128 * groups, smem, st, geo, mlp, ws, map, (const T*)feat, box.vb, box.vx, box_bytes, groups);
   }
   count_launches(1);
   e = cudaGetLastError();
@@ -838,7 +857,7 @@ static cicero_status launch_tc_hash(const GridGeo& geo, const MlpPtrs& mlp, cons
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(k_gather_mlp_bf16_hash)");
   {
     ProfScope ps(kStGatherMlp, st);
-    kern<<<num_sms(), 128 * groups, smem, st>>>(geo, mlp, ws, hg, groups);
+    launch_kernel(kern, num_sms(), 128 * groups, smem, st, geo, mlp, ws, hg, groups);
   }
   count_launches(1);
   e = cudaGetLastError();
@@ -869,7 +888,7 @@ static cicero_status launch_tc_batch(const BatchPlan& b, int groups, cudaStream_
   }
   {
     ProfScope ps(kStGatherMlp, st);
-    kern<<<num_sms(), 128 * groups, smem, st>>>(b.jobs, b.n_jobs, b.ws, b.box.vb, b.box.vx, box_bytes, groups);
+    launch_kernel(kern, num_sms(), 128 * groups, smem, st, b.jobs, b.n_jobs, b.ws, b.box.vb, b.box.vx, box_bytes, groups);
   }
   count_launches(1);
   e = cudaGetLastError();
@@ -900,7 +919,7 @@ cicero_status launch_mlp_eval_bf16(const MlpPtrs& mlp, const float* x, int M, fl
   const int grid = std::max(1, std::min((ntile + kMaxGroups - 1) / kMaxGroups, num_sms()));
   {
     ProfScope ps(kStMlpEval, st);
-    k_mlp_eval_bf16<<<grid, 128 * kMaxGroups, smem, st>>>(mlp, x, M, c, err);
+    launch_kernel(k_mlp_eval_bf16, grid, 128 * kMaxGroups, smem, st, mlp, x, M, c, err);
   }
   count_launches(1);
   e = cudaGetLastError();

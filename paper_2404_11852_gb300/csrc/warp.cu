@@ -5,8 +5,8 @@
 //                  Eq. 3 (projection) and the depth test as one 64-bit atomicMin of
 //                  (float bits of Z') << 32 | reference index
 //   W3 k_resolve   per target pixel: copy the winner's colour, or classify the hole (void when
-//                  its ray has no sample in the grid box / occupied cells)
-//   W4 k_hole_*    stream compaction of the holes in ascending pixel order (block scans)
+//                  its ray has no sample in the grid box / occupied cells); holes per chunk
+//   W4 k_hole_write  stream compaction of the holes in ascending pixel order
 // All decision arithmetic uses explicit round-to-nearest intrinsics (no FMA contraction).
 #include <cuda_runtime.h>
 
@@ -79,12 +79,16 @@ __device__ __forceinline__ Splat splat_point(const WarpArgs& a, const float* ref
 // Kernels take the whole batch of target views as a __grid_constant__ parameter; blockIdx.y is
 // the view.
 __global__ void k_zclear(const __grid_constant__ WarpBatch B) {
+  dependents_sync();
   const WarpView& V = B.v[blockIdx.y];
   const int n = V.a.wt * V.a.ht;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) V.z[i] = ~0ull;
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x, st = gridDim.x * blockDim.x;
+  for (int i = i0; i < n; i += st) V.z[i] = ~0ull;
+  for (int i = i0; i < V.nblk; i += st) V.bsum[i] = 0;  // holes per chunk, counted by k_resolve
 }
 
 __global__ void __launch_bounds__(256) k_splat(const __grid_constant__ WarpBatch B, const float* __restrict__ ref_depth) {
+  dependents_sync();
   const WarpView& V = B.v[blockIdx.y];
   const int n = V.a.wr * V.a.hr;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
@@ -119,17 +123,26 @@ __device__ __forceinline__ bool warp_ray_has_sample(const VoidTest& vt, const fl
   return false;
 }
 
-// One warp per 32 consecutive target pixels: copy the winners, mark the holes (3 = still to be
-// tested for void when the void test is on, else 1).
+// Hole compaction: bsum holds the holes of each kHoleChunk consecutive pixels of a view.
+constexpr int kHoleChunk = 4096;
+constexpr int kResolvePix = 1024;  // pixels per block of k_resolve
+
+// Copy the winners, mark the holes (3 = still to be tested for void when the void test is on, else 1)
+// and count them per chunk (a block's pixels lie in one chunk).
 __global__ void __launch_bounds__(256) k_resolve(const __grid_constant__ WarpBatch B, int void_on,
                                                  const float* __restrict__ ref_rgb, const float* __restrict__ ref_depth) {
+  dependents_sync();
+  static_assert(kHoleChunk % kResolvePix == 0, "a block's pixels lie in one chunk");
   const WarpView& V = B.v[blockIdx.y];
   const int n = V.a.wt * V.a.ht;
-  const int lane = threadIdx.x & 31;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int p0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; p0 < n; p0 += nwarps * 32) {
-    const int p = p0 + lane;
-    if (p >= n) continue;
+  __shared__ uint32_t holes;
+  if (threadIdx.x == 0) holes = 0;
+  __syncthreads();
+  uint32_t mine = 0;
+#pragma unroll
+  for (int k = 0; k < kResolvePix / 256; k++) {
+    const int p = blockIdx.x * kResolvePix + k * 256 + threadIdx.x;
+    if (p >= n) break;
     const unsigned long long key = V.z[p];
     if (key != ~0ull) {
       const int q = (int)(key & 0xffffffffull);
@@ -148,8 +161,14 @@ __global__ void __launch_bounds__(256) k_resolve(const __grid_constant__ WarpBat
       V.wrgb[3 * p + 2] = 0.0f;
       if (V.wdepth) V.wdepth[p] = 0.0f;
       V.mask[p] = void_on ? 3 : 1;
+      mine++;
     }
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&holes, mine);
+  __syncthreads();
+  if (threadIdx.x == 0 && holes) atomicAdd(&V.bsum[blockIdx.x / (kHoleChunk / kResolvePix)], holes);
 }
 
 // Per-candidate setup shared by a warp: the target ray and its slots.
@@ -164,6 +183,7 @@ struct VoidSetup {
 // i = warp + k nwarps; lane j prepares the ray and slots of the j-th of each group of 32 of them,
 // which the whole warp then reads from shared memory candidate by candidate.
 __global__ void __launch_bounds__(256) k_void(const __grid_constant__ WarpBatch B, const __grid_constant__ VoidTest vt) {
+  dependents_sync();
   const int v = blockIdx.y;
   const WarpView& V = B.v[v];
   const int lane = threadIdx.x & 31;
@@ -216,6 +236,7 @@ __global__ void __launch_bounds__(256) k_void(const __grid_constant__ WarpBatch 
           V.wrgb[3 * p + 2] = vt.s.bg[2];
           if (V.wdepth) V.wdepth[p] = __int_as_float(0x7f800000);
           V.mask[p] = 2;
+          atomicSub(&V.bsum[p / kHoleChunk], 1u);  // no longer a hole of its chunk
         } else {
           V.mask[p] = 1;
         }
@@ -224,9 +245,6 @@ __global__ void __launch_bounds__(256) k_void(const __grid_constant__ WarpBatch 
     __syncwarp();  // the setup slots are free for the next group
   }
 }
-
-// Hole compaction: each block of 1024 threads owns kHoleChunk consecutive pixels of its view.
-constexpr int kHoleChunk = 4096;
 
 __device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t* tot, uint32_t* sh) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -254,41 +272,18 @@ __device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t* tot, uint
   return r;
 }
 
-__global__ void __launch_bounds__(1024) k_hole_count(const __grid_constant__ WarpBatch B, uint8_t val) {
+// The holes (mask == val) in ascending pixel order: each block of 1024 threads owns one chunk, adds up the
+// counts of the chunks before it and lists its own; the view's last block writes the total.  (Counting in
+// k_resolve and the sum here replace a counting and a scan kernel each time.)
+__global__ void __launch_bounds__(1024) k_hole_write(const __grid_constant__ WarpBatch B, uint8_t val) {
+  dependents_sync();
   __shared__ uint32_t sh[32];
   const WarpView& V = B.v[blockIdx.y];
   if ((int)blockIdx.x >= V.nblk) return;  // uniform per block
   const int n = V.a.wt * V.a.ht;
   const int base = blockIdx.x * kHoleChunk + threadIdx.x * 4;
-  uint32_t c = 0;
-#pragma unroll
-  for (int k = 0; k < 4; k++) c += (base + k < n && V.mask[base + k] == val) ? 1u : 0u;
-  uint32_t tot;
-  block_exscan(c, &tot, sh);
-  if (threadIdx.x == 0) V.bsum[blockIdx.x] = tot;
-}
-
-__global__ void __launch_bounds__(1024) k_hole_blocks(const __grid_constant__ WarpBatch B) {
-  __shared__ uint32_t sh[32];
-  const WarpView& V = B.v[blockIdx.y];
-  uint32_t run = 0;
-  for (int b0 = 0; b0 < V.nblk; b0 += blockDim.x) {
-    const int i = b0 + threadIdx.x;
-    const uint32_t x = i < V.nblk ? V.bsum[i] : 0;
-    uint32_t tot;
-    const uint32_t e = block_exscan(x, &tot, sh);
-    if (i < V.nblk) V.bsum[i] = run + e;
-    run += tot;
-  }
-  if (threadIdx.x == 0) *V.n_holes = (int32_t)run;
-}
-
-__global__ void __launch_bounds__(1024) k_hole_write(const __grid_constant__ WarpBatch B, uint8_t val) {
-  __shared__ uint32_t sh[32];
-  const WarpView& V = B.v[blockIdx.y];
-  if ((int)blockIdx.x >= V.nblk) return;
-  const int n = V.a.wt * V.a.ht;
-  const int base = blockIdx.x * kHoleChunk + threadIdx.x * 4;
+  uint32_t before = 0;
+  for (int i = threadIdx.x; i < (int)blockIdx.x; i += blockDim.x) before += V.bsum[i];
   uint32_t c = 0;
   bool h[4];
 #pragma unroll
@@ -296,18 +291,20 @@ __global__ void __launch_bounds__(1024) k_hole_write(const __grid_constant__ War
     h[k] = base + k < n && V.mask[base + k] == val;
     c += h[k] ? 1u : 0u;
   }
-  uint32_t tot;
-  uint32_t pos = V.bsum[blockIdx.x] + block_exscan(c, &tot, sh);
+  uint32_t tot, run;
+  block_exscan(before, &run, sh);
+  uint32_t pos = run + block_exscan(c, &tot, sh);
 #pragma unroll
   for (int k = 0; k < 4; k++)
     if (h[k]) V.hole_idx[pos++] = base + k;
+  if ((int)blockIdx.x == V.nblk - 1 && threadIdx.x == 0) *V.n_holes = (int32_t)(run + tot);
 }
 
 // Bilinear resampling of an image (the DS-2 comparator of the evaluation: render at half resolution,
 // then upsample).  Pixel centres align: output pixel i samples the source at u = (i + 1/2) w / W - 1/2,
 // interpolating the two nearest source pixel centres per axis, clamped to the image.
-__global__ void __launch_bounds__(256) k_upsample(const float* __restrict__ src, int w, int h, int C,
-                                                  float* __restrict__ dst, int W, int H) {
+__global__ void __launch_bounds__(256) k_upsample(const float* src, int w, int h, int C, float* dst, int W, int H) {
+  dependents_sync();
   const long long n = (long long)W * H;
   const float sx = (float)w / (float)W, sy = (float)h / (float)H;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
@@ -331,7 +328,7 @@ __global__ void __launch_bounds__(256) k_upsample(const float* __restrict__ src,
 cicero_status run_upsample(const float* src, int w, int h, int C, float* dst, int W, int H, cudaStream_t st) {
   const long long n = (long long)W * H;
   const int blocks = (int)std::min<long long>((n + 255) / 256, (long long)num_sms() * 8);
-  k_upsample<<<blocks, 256, 0, st>>>(src, w, h, C, dst, W, H);
+  launch_kernel(k_upsample, blocks, 256, 0, st, src, w, h, C, dst, W, H);
   count_launches(1);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? CICERO_OK : cuda_fail(e, "k_upsample");
@@ -374,27 +371,23 @@ cicero_status run_warp(const WarpBatch& B, const VoidTest& vt, const float* ref_
   const int nr = B.v[0].a.wr * B.v[0].a.hr;
   const int g = std::max(1, num_sms() * 8 / B.n_views);
   const dim3 gz(std::min(g, (max_nt + 255) / 256), B.n_views), gs(std::min(g, (nr + 255) / 256), B.n_views);
-  const dim3 gb(max_blk, B.n_views), g1(1, B.n_views), gv(g, B.n_views);
+  const dim3 gb(max_blk, B.n_views), gv(g, B.n_views), gr((max_nt + kResolvePix - 1) / kResolvePix, B.n_views);
   {
     ProfScope ps(kStWarpSplat, st);
-    k_zclear<<<gz, 256, 0, st>>>(B);
-    k_splat<<<gs, 256, 0, st>>>(B, ref_depth);
+    launch_kernel(k_zclear, gz, 256, 0, st, B);
+    launch_kernel(k_splat, gs, 256, 0, st, B, ref_depth);
   }
   {
     ProfScope ps(kStWarpResolve, st);
-    k_resolve<<<gz, 256, 0, st>>>(B, vt.enabled, ref_rgb, ref_depth);
+    launch_kernel(k_resolve, gr, 256, 0, st, B, vt.enabled, ref_rgb, ref_depth);
     if (vt.enabled) {  // list the candidates, test them, then list the holes that remain
-      k_hole_count<<<gb, 1024, 0, st>>>(B, 3);
-      k_hole_blocks<<<g1, 1024, 0, st>>>(B);
-      k_hole_write<<<gb, 1024, 0, st>>>(B, 3);
-      k_void<<<gv, 256, 0, st>>>(B, vt);
-      count_launches(4);
+      launch_kernel(k_hole_write, gb, 1024, 0, st, B, 3);
+      launch_kernel(k_void, gv, 256, 0, st, B, vt);
+      count_launches(2);
     }
-    k_hole_count<<<gb, 1024, 0, st>>>(B, 1);
-    k_hole_blocks<<<g1, 1024, 0, st>>>(B);
-    k_hole_write<<<gb, 1024, 0, st>>>(B, 1);
+    launch_kernel(k_hole_write, gb, 1024, 0, st, B, 1);
   }
-  count_launches(6);
+  count_launches(4);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? CICERO_OK : cuda_fail(e, "warp kernels");
 }

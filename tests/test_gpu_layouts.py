@@ -119,3 +119,63 @@ def test_backward_masks_and_fixup(cc, orc, C, dtype, with_mlp):
         if a is not None:
             a = a.cpu().double().numpy().ravel()
             assert np.abs(a - np.ravel(b)).max() <= 1e-4 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("N,brick,side", [(9, 4, 7), (33, 4, 40), (66, 4, 33), (130, 4, 24)])
+def test_ray_index_table_scan(cc, N, brick, side):
+    """The table from one scan block (1024 bricks) to several dozen, and tiles that end inside a brick:
+    offsets and samples are consistent, and every sample of a brick appears once."""
+    import torch
+    g = scenes.make_grid(N, 4, 3, seed=900 + N)
+    cam = scenes.orbit_camera(side, side, az_deg=35.0, sampling=scenes.sampling_uniform(64, t_stop=0.0))
+    gd, cd, sd = cc.DeviceGrid.from_host(g), cc.camera_from(cam), cc.sampling_from(cam.sampling)
+    opt = cc.options(cc.MLP_FP32, brick)
+    nb = (-(-(N - 1) // brick)) ** 3
+    offs = torch.full((nb + 1,), -1, dtype=torch.int32, device="cuda")
+    smp = torch.full((side * side * 64,), -1, dtype=torch.int32, device="cuda")
+    ws = cc.workspace(cc.cicero_build_rit_workspace_size(gd.desc, cd, sd, opt))
+    assert cc.cicero_build_rit(gd.desc, cd, sd, opt, offs, smp, ws) == nb
+    cc.cicero_workspace_status(ws)
+    o, n = offs.cpu().numpy(), None
+    hdr = ws[:16].view(torch.int32).cpu().numpy()
+    n = int(hdr[2])
+    assert o[0] == 0 and o[-1] == n and (np.diff(o) >= 0).all()
+    assert int(hdr[1]) == int((-(-np.diff(o) // 128)).sum())  # tiles
+    got = smp.cpu().numpy()[:n]
+    assert len(np.unique(got)) == n and got.min() >= 0
+    # the brick of each sample, from its position in FP64; samples within rounding of a face may differ
+    ray, slot = got // 64, got % 64
+    c2w = cam.c2w.astype(np.float64)
+    u = np.stack([(ray % side + 0.5 - cam.cx) / cam.f, (ray // side + 0.5 - cam.cy) / cam.f, np.ones(n)], 1)
+    d = u @ c2w[:, :3].T
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    p = c2w[:, 3] + (0.5 + (slot + 0.5) * (2.0 / 64))[:, None] * d
+    v = np.minimum(np.floor((p + 1.0) * 0.5 * (N - 1)), N - 2).astype(int) // brick
+    k = -(-(N - 1) // brick)
+    want = (v[:, 2] * k + v[:, 1]) * k + v[:, 0]
+    assert (want == np.repeat(np.arange(nb), np.diff(o))).mean() > 0.999
+
+
+@pytest.mark.parametrize("w,h,void", [(1, 1, True), (37, 29, False), (64, 64, True), (129, 130, True), (4096, 3, False)])
+def test_warp_hole_list(cc, orc, w, h, void):
+    """Hole counting and listing from a single chunk of 4096 pixels to several, ragged ones among them."""
+    import torch
+    cam = scenes.orbit_camera(w, h, az_deg=10.0, sampling=scenes.sampling_uniform(32))
+    tgt = scenes.offset_camera(cam, 3)
+    g = scenes.make_grid(24, 4, 3, seed=950)
+    rng = np.random.default_rng(w * h)
+    rgb = rng.random((w * h, 3), dtype=np.float32)
+    depth = np.where(rng.random(w * h) < 0.3, np.inf, 1.0 + 0.3 * rng.random(w * h)).astype(np.float32)
+    want = orc.warp(rgb, depth, cam, tgt, void_grid=g if void else None, void_sampling=cam.sampling if void else None)
+    gd, sd = cc.DeviceGrid.from_host(g), cc.sampling_from(cam.sampling)
+    out = [torch.empty(w * h, 3, device="cuda"), torch.empty(w * h, device="cuda"),
+           torch.empty(w * h, dtype=torch.uint8, device="cuda"), torch.empty(w * h, dtype=torch.int32, device="cuda"),
+           torch.empty(1, dtype=torch.int32, device="cuda")]
+    tc = cc.camera_from(tgt)
+    cc.cicero_warp(torch.from_numpy(rgb).cuda(), torch.from_numpy(depth).cuda(), cc.camera_from(cam), tc, 180.0,
+                   gd.desc if void else None, sd if void else None, *out, cc.workspace(cc.cicero_warp_workspace_size(tc)))
+    assert (out[2].cpu().numpy() == want["mask"]).all()
+    n = int(out[4].item())
+    assert n == want["n_holes"]
+    assert (out[3].cpu().numpy()[:n] == np.flatnonzero(want["mask"] == 1)).all()
+    assert (out[0].cpu().numpy() == want["rgb"].astype(np.float32)).all()
