@@ -647,6 +647,19 @@ __device__ __forceinline__ void block_exscan2(uint32_t a, uint32_t b, uint32_t* 
   __syncthreads();
 }
 
+// Where a key's scatter cursor stands.  The cursors of neighbouring bricks share 128-byte lines, and a
+// line's atomics all go to one L2 slice: on a small scene whose samples lie in a few hundred bricks one
+// slice took 8 times the average (60% busy, the others 4%).  From 1025 to 16384 bricks the cursors are
+// spread: octant by octant, neighbouring bricks cursor_step entries apart (bucketing of a 64^3 scene with bricks of 4,
+// 400x304: 199 -> 163 us a frame; of 2,100 bricks 266 -> 260).  Larger tables spread by themselves and gain
+// more from a ray's consecutive keys lying together (256^3, bricks of 4: 643 -> 702 us spread).
+__device__ __forceinline__ uint32_t cursor_step(uint32_t nb) {  // coprime to nb (a prime that does not divide it)
+  return nb <= 1024u || nb > 16384u ? 0u : (nb % 1009u ? 1009u : 1013u);
+}
+__device__ __forceinline__ uint32_t cursor_at(uint32_t key, uint32_t nb, uint32_t step) {
+  return step ? (key % kOctants) * nb + ((key / kOctants) * step) % nb : key;
+}
+
 // The kOctants counters of brick b (zeros past the last brick).
 __device__ __forceinline__ uint32_t brick_counts(const RenderWs& w, int b, uint32_t v[kOctants]) {
   static_assert(kOctants == 8, "two 16-byte loads per brick");
@@ -682,7 +695,8 @@ __global__ void __launch_bounds__(1024) k_brick_sums(RenderWs w) {
 // block K2a is not launched.  (Two kernels fewer than a scan of the block sums and a kernel of tiles that
 // searched all bricks' offsets in global memory: scan and tiles of the 800x800 frame 38 -> 28 us, a 64x64
 // frame's bucketing 27 -> 17.)
-// BATCH: bricks are numbered job after job.
+// With few bricks of many tiles each, gridDim.y blocks repeat a chunk's scan and share its tiles (3 blocks
+// alone took 48 us for 144 K tiles).  BATCH: bricks are numbered job after job.
 template <bool BATCH>
 __global__ void __launch_bounds__(1024) k_brick_offsets(GridGeo g, const JobDesc* __restrict__ jobs,
                                                         const int* __restrict__ bases, int n_jobs, RenderWs w) {
@@ -705,7 +719,7 @@ __global__ void __launch_bounds__(1024) k_brick_offsets(GridGeo g, const JobDesc
   first_tile[threadIdx.x] = et;
   first[threadIdx.x] = base_c + ec;
   count[threadIdx.x] = c;
-  if (b < w.nb) {
+  if (b < w.nb && blockIdx.y == 0) {
     uint32_t o[kOctants], run = base_c + ec;
 #pragma unroll
     for (int k = 0; k < kOctants; k++) {
@@ -715,12 +729,18 @@ __global__ void __launch_bounds__(1024) k_brick_offsets(GridGeo g, const JobDesc
     uint4* off = reinterpret_cast<uint4*>(w.brick_off + (size_t)b * kOctants);
     off[0] = make_uint4(o[0], o[1], o[2], o[3]);
     off[1] = make_uint4(o[4], o[5], o[6], o[7]);
-    uint4* cur = reinterpret_cast<uint4*>(w.brick_cur + (size_t)b * kOctants);  // cursors start at the offsets
-    cur[0] = make_uint4(o[0], o[1], o[2], o[3]);
-    cur[1] = make_uint4(o[4], o[5], o[6], o[7]);
+    const uint32_t step = cursor_step((uint32_t)w.nb);
+    if (step) {
+#pragma unroll
+      for (int k = 0; k < kOctants; k++) w.brick_cur[cursor_at((uint32_t)b * kOctants + k, (uint32_t)w.nb, step)] = o[k];
+    } else {
+      uint4* cur = reinterpret_cast<uint4*>(w.brick_cur + (size_t)b * kOctants);  // cursors start at the offsets
+      cur[0] = make_uint4(o[0], o[1], o[2], o[3]);
+      cur[1] = make_uint4(o[4], o[5], o[6], o[7]);
+    }
     w.tile_off[b] = base_t + et;
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+  if (blockIdx.x == gridDim.x - 1 && blockIdx.y == 0 && threadIdx.x == 0) {
     uint32_t run_t = base_t + tt;
     w.brick_off[(size_t)w.nb * kOctants] = base_c + tc;
     w.tile_off[w.nb] = run_t;
@@ -732,7 +752,8 @@ __global__ void __launch_bounds__(1024) k_brick_offsets(GridGeo g, const JobDesc
     w.hdr[2] = base_c + tc;
   }
   __syncthreads();
-  for (uint32_t q = threadIdx.x; q < tt && base_t + q < (uint32_t)w.max_tiles; q += blockDim.x) {
+  for (uint32_t q = blockIdx.y * blockDim.x + threadIdx.x; q < tt && base_t + q < (uint32_t)w.max_tiles;
+       q += gridDim.y * blockDim.x) {
     int lo = 0;  // the last brick of the block whose first tile is <= q
 #pragma unroll
     for (int step = kScanChunk / 2; step > 0; step >>= 1)
@@ -767,6 +788,7 @@ __global__ void __launch_bounds__(256, 4) k_scatter(RaySrc src, RenderWs w) {
   const unsigned full = 0xffffffffu;
   const unsigned lt_mask = (1u << lane) - 1u;
   const unsigned le_mask = (2u << lane) - 1u;
+  const uint32_t cstep = cursor_step((uint32_t)w.nb);
   struct Chunk {
     uint32_t key, slot;
     float wk;
@@ -836,7 +858,7 @@ __global__ void __launch_bounds__(256, 4) k_scatter(RaySrc src, RenderWs w) {
         const unsigned after = heads & ~le_mask;
         const int end = after ? __ffs(after) - 1 : 32;
         const unsigned run = vmask & ~lt_mask & (end == 32 ? full : ((1u << end) - 1u));
-        off = atomicAdd(&w.brick_cur[c.key], (uint32_t)__popc(run));
+        off = atomicAdd(&w.brick_cur[cursor_at(c.key, (uint32_t)w.nb, cstep)], (uint32_t)__popc(run));
       }
       // the previous chunk is written while this chunk's atomics are in flight
       flush();
@@ -1399,6 +1421,9 @@ static int setup_blocks(long long rays) {
   return (int)std::max(1ll, std::min((rays + 255) / 256, (long long)num_sms() * 8));
 }
 
+// K2b: the scan's blocks, and as many for each as fill the SMs once
+static dim3 offset_grid(int nblk) { return dim3(nblk, std::max(1, num_sms() / nblk)); }
+
 static int blocks_for_warps(long long warps, int per_sm) {
   long long blocks = (warps + 7) / 8;
   long long cap = (long long)num_sms() * per_sm;
@@ -1438,7 +1463,7 @@ cicero_status run_render(const cicero_grid* grid, const MlpPtrs& mlp, const Rend
     ProfScope ps(kStBucket, st);
     const int nblk = (plan.nb + kScanChunk - 1) / kScanChunk;
     if (nblk > 1) launch_kernel(k_brick_sums, nblk, 1024, 0, st, ws);
-    launch_kernel(k_brick_offsets<false>, nblk, 1024, 0, st, geo, nullptr, nullptr, 0, ws);
+    launch_kernel(k_brick_offsets<false>, offset_grid(nblk), 1024, 0, st, geo, nullptr, nullptr, 0, ws);
     count_launches(nblk > 1 ? 6 : 5);
     launch_kernel(k_scatter, mb, 256, 0, st, src, ws);
   }
@@ -1504,7 +1529,7 @@ cicero_status run_render_batch(const BatchPlan& b, cudaStream_t st) {
     ProfScope ps(kStBucket, st);
     const int nblk = (plan.nb + kScanChunk - 1) / kScanChunk;
     if (nblk > 1) launch_kernel(k_brick_sums, nblk, 1024, 0, st, ws);
-    launch_kernel(k_brick_offsets<true>, nblk, 1024, 0, st, plan.geo, b.jobs, b.bases, b.n_jobs, ws);
+    launch_kernel(k_brick_offsets<true>, offset_grid(nblk), 1024, 0, st, plan.geo, b.jobs, b.bases, b.n_jobs, ws);
     count_launches(nblk > 1 ? 6 : 5);
     launch_kernel(k_scatter, mb, 256, 0, st, src, ws);
   }
