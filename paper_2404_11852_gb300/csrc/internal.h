@@ -95,6 +95,7 @@ struct RenderWs {
   SrtRec* srt;          // [Q] the Ray Index Table payload in brick order
   RayGeo* ray_geo;      // [R] geometry of each ray's samples
   struct RaySetup* setup;  // [R] per-ray setup of the march (ray, slots, active-slot mask, records)
+  void* pack;           // [n2][n1][n0] voxels of eight FP16 corner densities (k_pack), or NULL
   char* stage;          // per-sample operands of the MLP weight gradients (backward with d_mlp only; may be
                         // null): blocks of kStageBlock sorted samples, WgStage::bytes each (stage_col)
   int R, S, nb, max_tiles;
@@ -129,6 +130,7 @@ struct RenderPlan {
   uint32_t Q;
   bool want_k;
   bool want_bwd;
+  size_t pack_bytes;  // of the packed voxels (RenderWs::pack); 0 = the march reads the density array itself
   bool want_wg;  // the backward stages the MLP weight gradients' operands (RenderWs::stage)
   cicero_precision precision;
   int mlp_groups;  // BF16 tensor-core MLP tiles in flight per SM (0 = as many as fit)

@@ -179,3 +179,38 @@ def test_warp_hole_list(cc, orc, w, h, void):
     assert n == want["n_holes"]
     assert (out[3].cpu().numpy()[:n] == np.flatnonzero(want["mask"] == 1)).all()
     assert (out[0].cpu().numpy() == want["rgb"].astype(np.float32)).all()
+
+
+@pytest.mark.parametrize("n,occ,precision", [((2, 2, 2), 0, 1), ((6, 3, 35), 0, 0), ((34, 17, 9), 5, 1),
+                                             ((18, 40, 33), 64, 1), ((66, 33, 20), 16, 2), ((50, 51, 52), 1, 0)])
+def test_packed_density_is_the_same(cc, n, occ, precision):
+    """The march over packed voxels (k_pack) gives the bits of the march over the density array, which a
+    workspace without room for the voxels takes: odd sizes, cells larger and smaller than voxels."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(sum(n) + occ)
+    dens = (torch.rand((n[2], n[1], n[0]), generator=gen, device="cuda") * 12 - 4).half()
+    feat = (torch.rand((n[2], n[1], n[0], 4), generator=gen, device="cuda") * 2 - 1).half()
+    mask = (torch.rand((occ,) * 3, generator=gen, device="cuda") < 0.4).to(torch.uint8) if occ else None
+    g, m = cc.DeviceGrid(dens, feat, occ=mask), cc.DeviceMlp.from_host(scenes.make_mlp(4, seed=3))
+    cam = scenes.orbit_camera(90, 61, az_deg=33.0)
+    cd, opt = cc.camera_from(cam), cc.options(precision, 4)
+    R = 90 * 61
+    for sd in (cc.sampling(0.5, 2.5, 300, 0.0, 1e-3), cc.sampling(0.0, 1e30, 120, 0.03, 0.0)):
+        need = cc.cicero_render_workspace_size(g.desc, R, sd, opt)
+        out = []
+        for bytes_ in (need, need - 256):
+            ws = cc.workspace(bytes_)
+            o = [torch.empty(R, 3, device="cuda"), torch.empty(R, device="cuda"), torch.empty(R, device="cuda"),
+                 torch.empty(R, dtype=torch.int32, device="cuda")]
+            cc.cicero_profile_begin()
+            n0 = cc.cicero_launch_count()
+            cc.cicero_render(g.desc, m.desc, cd, sd, opt, *o, ws)
+            launches = cc.cicero_launch_count() - n0
+            cc.cicero_profile_end()
+            cc.cicero_workspace_status(ws)
+            out.append((launches, o))
+        assert out[0][0] == out[1][0] + 1  # one kernel more: the packing
+        for a, b in zip(out[0][1], out[1][1]):
+            assert torch.equal(a, b)
+        with pytest.raises(cc.CiceroError):  # without the voxels the workspace may not shrink any further
+            cc.cicero_render(g.desc, m.desc, cd, sd, opt, *out[0][1], cc.workspace(need - 512 - 16 * n[0] * n[1] * n[2]))
