@@ -48,18 +48,8 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
       : "memory");
 }
 
-// the same with A read from tensor memory (row m = lane m, two BF16 K values per 32-bit column)
-__device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc,
-                                            uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-
-// The same MMAs for a warp that runs them with warp-uniform operands (one elected lane inside the
+// The same MMA, and the one with A read from tensor memory (row m = lane m, two BF16 K values per
+// 32-bit column), for a warp that runs them with warp-uniform operands (one elected lane inside the
 // branch): the descriptors as their low words (address and leading byte offset) and, constant, their high
 // words (stride byte offset and version), so that a K step further is one 32-bit addition that the
 // compiler keeps in uniform registers, where the instruction reads its operands.
