@@ -362,15 +362,17 @@ __global__ void __launch_bounds__(256) k_pack(GridGeo g, const __half* __restric
   const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 8 + (threadIdx.x >> 5);
   if (x >= g.n[0] - 1 || y >= g.n[1] - 1) return;
   const size_t nx = g.n[0], nxy = nx * g.n[1];
-  // the occupancy cells that a position inside the voxel can fall into, a rounding apart
+  // the occupancy cells that a position inside the voxel can fall into, a rounding apart: at most three an
+  // axis, and where cells are smaller than voxels (any number in one) all voxels are packed
   const int R = g.occ_res;
+  const bool masked = g.occ && R < min(g.n[0], min(g.n[1], g.n[2]));
   const float eps = 1e-3f + 1e-6f * (float)R;
   auto cells = [&](int a, int i, int& lo, int& hi) {
     lo = max(0, min(R - 1, (int)floorf((float)i * g.occ_scale[a] - eps)));
     hi = max(0, min(R - 1, (int)floorf((float)(i + 1) * g.occ_scale[a] + eps)));
   };
   int x_lo = 0, x_hi = 0, y_lo = 0, y_hi = 0, z_lo = -1, z_hi = -1;
-  if (g.occ) {
+  if (masked) {
     cells(0, x, x_lo, x_hi);
     cells(1, y, y_lo, y_hi);
   }
@@ -379,7 +381,7 @@ __global__ void __launch_bounds__(256) k_pack(GridGeo g, const __half* __restric
   const unsigned short* d = reinterpret_cast<const unsigned short*>(dens);
   const int z1 = min((int)(blockIdx.z + 1) * kPackZ, g.n[2] - 1);
   for (int z = blockIdx.z * kPackZ; z < z1; z++) {
-    if (g.occ) {
+    if (masked) {
       int lo, hi;
       cells(2, z, lo, hi);
       if (lo != z_lo || hi != z_hi) {
