@@ -520,7 +520,7 @@ def batched_workload(cc, torch, dev, n_check=8, reps=5):
             "batch_ms": t_batch,
             "jobs_per_s": BATCH_JOBS / (t_batch / 1e3), "msamples_per_s": samples / (t_batch / 1e3) / 1e6,
             "one_call_per_job_ms": t_single, "speedup_vs_one_call_per_job": t_single / t_batch,
-            "launch": "one CUDA graph (10 kernels for all jobs)", "record_capacity": cap, "stage_ms": stage_ms,
+            "launch": "one CUDA graph (8 kernels for all jobs)", "record_capacity": cap, "stage_ms": stage_ms,
             "oracle_check": {"pixels": n // 3, "max_err": worst, "psnr_db": 10 * math.log10(1.0 / max(sq / n, 1e-30))}}
 
 
@@ -729,7 +729,7 @@ def backward_workload(cc, torch, dev):
     cc.cicero_workspace_status(ws_b)
     hdr = ws_b[:32].view(torch.int32).cpu().numpy()
     samples = int(hdr[2])  # composited samples of the recompute
-    fixed = int(hdr[4])    # of which recomputed in FP32 (uncertain split-BF16 ReLU decisions)
+    fixed = int(hdr[4])    # of which recomputed in FP32 (uncertain ReLU decisions)
     # per-stage device time of one backward call without and with the MLP weight gradients
     stage = {}
     for name, arg, ws in (("grid", None, None), ("grid_and_mlp", dm, ws_bm), ("grid_and_mlp_cuda_cores", dm, None)):
