@@ -47,7 +47,10 @@ typedef enum { CICERO_F32 = 0, CICERO_F16 = 1 } cicero_dtype;
 /* Arithmetic of Feature Computation (the MLP):
  * FP32: the accuracy of FP32.  cicero_mlp_eval runs FP32 FFMA on CUDA cores; the rendering calls split
  * every operand of layers 1 and 2 into three BF16 parts (24 significand bits) and take the six products
- * above 2^-24 on the tensor cores with FP32 accumulation; biases, layer 3 and the sigmoid in FP32.  BF16: tcgen05 tensor-core MMAs with BF16 operands (weights and
+ * above 2^-24 on the tensor cores with FP32 accumulation; biases, layer 3 and the sigmoid in FP32.  A sample
+ * with operands that have no such parts (infinities, magnitudes that BF16 rounds to infinity, or above 2^100
+ * beside weights below 2^-109) is computed by FP32 FFMA instead, so that infinities and NaNs act as in FP32
+ * (a hidden unit of NaN is 0 behind its ReLU).  BF16: tcgen05 tensor-core MMAs with BF16 operands (weights and
  * activations rounded to BF16) and FP32 accumulation in tensor memory.  FP32_SPLIT: FP32-class
  * accuracy on the tensor cores: every FP32 operand v of layers 1 and 2 is split into
  * hi = bf16(v) and lo = bf16(v - hi), each product taken as hi.hi + hi.lo + lo.hi (the method of

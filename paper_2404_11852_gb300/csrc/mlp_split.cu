@@ -93,6 +93,8 @@ struct Bars {  // one phase per use, in tile order
   uint64_t hfull[2];       // partial ||h1||^2 of tile i written           (8 E1 warps, backward)
   uint64_t last;           // every MMA done                               (commit)
   uint32_t tmem;
+  uint32_t odd;            // what the weights ask for (Odd)
+  uint32_t marked;         // whether a sample is marked to be taken again
 };
 static_assert(sizeof(Bars) <= 8 * 32, "barrier block");
 
@@ -213,6 +215,81 @@ struct Tmem {
 };
 __device__ __forceinline__ uint32_t h1_col(int k, uint32_t i) { return k == 0 ? 64u * (i & 1) : 64u * (uint32_t)(k + 1); }
 
+// FP32 renders: an operand that is infinite, or that BF16 rounds to infinity, has NaN parts, and every unit of
+// the sample would come out as NaN, 0 behind the ReLU, where the FP32 chain has infinities, zeros or finite
+// values.  Such samples are marked in their record's colour and taken again by E2 (sample_f32) when it is done
+// with the CTA's tiles.  E1 lets a NaN of its first unit through the ReLU (all units are NaNs then: an input
+// that cannot be split), layer 2's sums carry it (or that of an h1 that cannot be split), and E2 carries it
+// into the colour.  A NaN among the weights or biases of a unit marks nothing: the unit is 0 in both chains and
+// is taken out of the operands (drop_nan_units).
+// A weight or a bias of layer 1 from kHuge on marks every sample.  One below kTiny has parts below BF16's smallest number and is off
+// by up to 2^-134, too little to count beside operands below kHuge; with such weights G and E1 mark the
+// samples of larger ones.
+// A render without any of these pays an instruction or two per thread and tile, and the look at the weights
+// (62.5 M samples 8.78 -> 8.85 ms, a 64x64 frame the same); a sample taken again costs an SM ~5,000 clocks.
+constexpr float kHuge = 0x1p100f, kTiny = 0x1p-109f;
+constexpr uint32_t kOddColour = 0x7FC0BABEu;  // a NaN that no arithmetic returns
+enum Odd : uint32_t { kOddNan = 1, kOddAll = 2, kOddTiny = 4 };
+__device__ __forceinline__ float relu_nan(float v) {
+  float r;
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(v));
+  return r;
+}
+template <int N>
+__device__ __forceinline__ bool any_huge(const float* v) {
+  float m = 0.0f;
+#pragma unroll
+  for (int k = 0; k < N; k++) m = fmaxf(m, fabsf(v[k]));
+  return m >= kHuge;
+}
+
+// What the parameters in shared memory ask for, by this thread's share of the weights' hi parts (pairs of BF16
+// numbers; a NaN or an infinity shows there) and of the biases and layer 3.
+template <int NP>
+__device__ __forceinline__ uint32_t odd_parameters(const char* sm) {
+  using S = Smem<NP>;
+  uint32_t top = 0u, low = 0xFFFFFFFFu;  // per half: the largest magnitude, and the smallest but 0, minus 1
+#pragma unroll
+  for (int k = 0; k < (kW1Bytes + kW2Bytes + 16 * kThreads - 1) / (16 * kThreads); k++) {
+    const int i = 16 * (threadIdx.x + k * kThreads);
+    if (i >= kW1Bytes + kW2Bytes) break;
+    const uint4 q = *(const uint4*)(sm + (i < kW1Bytes ? S::w1 + i : S::w2 - kW1Bytes + i));
+    const uint32_t v[4] = {q.x & 0x7FFF7FFFu, q.y & 0x7FFF7FFFu, q.z & 0x7FFF7FFFu, q.w & 0x7FFF7FFFu};
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      top = __vmaxu2(top, v[u]);
+      low = __vminu2(low, __vsub2(v[u], 0x00010001u));
+    }
+  }
+  const uint32_t hi = max(top & 0xFFFFu, top >> 16), lo = min(low & 0xFFFFu, low >> 16);
+  uint32_t f = (hi > 0x7F80u ? kOddNan : hi >= (__float_as_uint(kHuge) >> 16) ? kOddAll : 0u) |
+               (lo < (__float_as_uint(kTiny) >> 16) - 1u ? kOddTiny : 0u);
+  for (int i = threadIdx.x; i < 5 * kHidden; i += kThreads) {
+    const float v = ((const float*)(sm + S::b1))[i];
+    f |= (isnan(v) ? kOddNan : 0u) | (i < kHidden && fabsf(v) >= kHuge ? kOddAll : 0u);
+  }
+  return f;
+}
+
+// Zeros in place of the weights and the bias of every unit that has a NaN among them (layer 3 is left alone).
+template <int NP>
+__device__ __noinline__ void drop_nan_units(char* sm, const MlpPtrs mlp) {
+  using S = Smem<NP>;
+  for (int r = threadIdx.x; r < 2 * kHidden; r += kThreads) {
+    const int n = r % kHidden, in = r < kHidden ? mlp.in_dim : kHidden, K = r < kHidden ? kK1 : kHidden;
+    const float* row = (r < kHidden ? mlp.w1 : mlp.w2) + (size_t)n * in;
+    float* bias = r < kHidden ? (float*)(sm + S::b1) + n : (float*)(sm + S::l3) + 8 * (n >> 1) + (n & 1);
+    bool drop = isnan(*bias);
+    for (int k = 0; k < in; k++) drop |= isnan(row[k]);
+    if (!drop) continue;
+    *bias = 0.0f;
+    for (int p = 0; p < NP; p++)
+      for (int k = 0; k < K; k += 8)
+        *(uint4*)(sm + (r < kHidden ? S::w1 + p * kW1Bytes : S::w2 + p * kW2Bytes) + tc::kmaj_off(n, k, K)) =
+            make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+
 // Weights [rows][in] (FP32, global) into NP K-major operands of K columns (zeros from `in` on).
 template <int NP>
 __device__ __forceinline__ void load_weights(char* dst, int part_bytes, const float* w, int rows, int in, int K) {
@@ -306,6 +383,86 @@ __device__ __forceinline__ void encode(const float d[3], float* x) {
       s[a] = s2;
     }
   }
+}
+
+// The colour of one sample from the FP32 chain on the CUDA cores, by a whole warp: for samples whose
+// operands cannot be split.  Lane l holds inputs l and l + 32 and hidden units 4 l .. 4 l +
+// 3; every unit's sum runs over its inputs in order, one FMA each.
+__device__ __forceinline__ float3 sample_f32(const GridGeo& g, const MlpPtrs& mlp, const void* feat, int f16,
+                                             const SrtRec* rec, bool w_finite) {
+  constexpr unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  float x[2] = {0.0f, 0.0f};
+  {
+    const float4 pw = rec->pw, qd = rec->qd;
+    const float p[3] = {pw.x, pw.y, pw.z};
+    int i0[3];
+    float f[3];
+    const bool in = index_sample(g, p, i0, f);  // (a sample that this rejects has set the error word)
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const int k = lane + 32 * u;
+      if (k < g.C) {
+        if (!in) continue;
+#pragma unroll 1
+        for (int q = 0; q < 8; q++) {
+          const float wq = ((q & 1) ? f[0] : 1.f - f[0]) * (((q >> 1) & 1) ? f[1] : 1.f - f[1]) *
+                           ((q >> 2) ? f[2] : 1.f - f[2]);
+          const size_t at = (((size_t)(i0[2] + (q >> 2)) * g.n[1] + (i0[1] + ((q >> 1) & 1))) * g.n[0] + i0[0] +
+                             (q & 1)) * g.C + k;
+          x[u] = fmaf(wq, f16 ? __half2float(((const __half*)feat)[at]) : ((const float*)feat)[at], x[u]);
+        }
+      } else if (k < mlp.in_dim) {  // d, then sin/cos(2^j d) as encode has them
+        const int e = k - g.C, a = e % 3;
+        const float d = a == 0 ? qd.y : (a == 1 ? qd.z : qd.w);
+        float s, c;
+        sincosf(d, &s, &c);
+#pragma unroll 1
+        for (int j = e < 3 ? 0 : (e - 3) / 6; j > 0; j--) {
+          const float s2 = 2.0f * s * c;
+          c = 1.0f - 2.0f * s * s;
+          s = s2;
+        }
+        x[u] = e < 3 ? d : ((e / 3) & 1 ? s : c);
+      }
+    }
+  }
+  float h[4] = {0.f, 0.f, 0.f, 0.f}, z[4] = {0.f, 0.f, 0.f, 0.f};
+  const bool none = __any_sync(full, isnan(x[0]) || isnan(x[1]));  // then all units of layer 1 are NaN, h1 0
+  if (none) z[0] = z[1] = z[2] = z[3] = NAN;
+#pragma unroll 1
+  for (int k = 0; k < mlp.in_dim && !none; k++) {
+    const float v = __shfl_sync(full, k < 32 ? x[0] : x[1], k & 31);
+#pragma unroll
+    for (int u = 0; u < 4; u++) z[u] = fmaf(v, mlp.w1[(4 * lane + u) * mlp.in_dim + k], z[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < 4; u++) {
+    h[u] = fmaxf(z[u] + mlp.b1[4 * lane + u], 0.0f);
+    z[u] = 0.0f;
+  }
+#pragma unroll 1
+  for (int k4 = 0; k4 < kHidden / 4 && !(none && w_finite); k4++)  // (h1 = 0 otherwise)
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      const float v = __shfl_sync(full, h[j], k4);
+#pragma unroll
+      for (int u = 0; u < 4; u++) z[u] = fmaf(v, mlp.w2[(4 * lane + u) * kHidden + 4 * k4 + j], z[u]);
+    }
+  float o[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+  for (int u = 0; u < 4; u++) {
+    const float h2 = fmaxf(z[u] + mlp.b2[4 * lane + u], 0.0f);
+#pragma unroll
+    for (int c = 0; c < 3; c++) o[c] = fmaf(mlp.w3[c * kHidden + 4 * lane + u], h2, o[c]);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) o[c] += __shfl_xor_sync(full, o[c], off);
+    o[c] = sigmoid_f(o[c] + mlp.b3[c]);
+  }
+  return make_float3(o[0], o[1], o[2]);
 }
 
 // M: every MMA of the CTA's n tiles, by one warp: the control flow and the operands are the warp's, one
@@ -410,7 +567,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
                                                            int f16) {
   using namespace tc;
   using S = Smem<NP>;
-  constexpr bool HOLD = hold<OUT>();
+  constexpr bool HOLD = hold<OUT>(), ODD = NP == 3 && OUT == Out::Colour;
   using RG = Regs<HOLD>;
   extern __shared__ __align__(1024) char sm[];
   Bars& B = *(Bars*)(sm + S::bars);
@@ -460,6 +617,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
       mbar_init(&B.mfull[k], kGatWarps);
     }
     mbar_init(&B.last, 1);
+    B.odd = B.marked = 0u;
     fence_mbar_init();
   }
   fence_proxy_async();
@@ -470,6 +628,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
   fence_before();
   __syncthreads();
   fence_after();
+  if constexpr (ODD) {
+    const uint32_t f = odd_parameters<NP>(sm);
+    if (f) atomicOr(&B.odd, f);
+    __syncthreads();
+    if (B.odd & kOddNan) {
+      drop_nan_units<NP>(sm, mlp);
+      fence_proxy_async();
+      __syncthreads();
+    }
+  }
   if constexpr (OUT != Out::Colour) {
     if (wid == 0) {
       float q = 0.0f;
@@ -497,6 +665,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
     (void)m;
     (void)meta;
     bool alive = true;
+    const bool tiny = ODD && (B.odd & kOddTiny);
+    (void)tiny;
     for (uint32_t i = 0; i < n && alive; i++) {
       if (!(alive = warp_wait(&B.l1done[i & 1], (i >> 1) & 1, err))) break;
       uint32_t rid = 0xffffffffu, mw[2] = {0u, 0u}, unsure = 0u;
@@ -513,6 +683,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
       fence_after();
       float v[HOLD ? 64 : 32];
       if constexpr (HOLD) load_half(dcol + 128u * (i & 1) + lanes, h, v);
+      if constexpr (ODD) {
+        if (tiny && any_huge<64>(v)) v[0] = NAN;
+      }
 #pragma unroll
       for (int q4 = 0; q4 < 4; q4++) {  // 16 units at a time, 4 / kChunks of them per chunk
         if constexpr (!HOLD) {
@@ -528,7 +701,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
           const float* z = v + 16 * (HOLD ? q4 : q4 % 2) + 4 * q;
           const float2 u0 = add2(make_float2(z[0], z[1]), make_float2(b.x, b.y));
           const float2 u1 = add2(make_float2(z[2], z[3]), make_float2(b.z, b.w));
-          const float2 r0 = make_float2(fmaxf(u0.x, 0.0f), fmaxf(u0.y, 0.0f));
+          float2 r0 = make_float2(fmaxf(u0.x, 0.0f), fmaxf(u0.y, 0.0f));
+          if constexpr (ODD) {
+            if (q4 == 0 && q == 0) r0.x = relu_nan(u0.x);
+          }
           const float2 r1 = make_float2(fmaxf(u1.x, 0.0f), fmaxf(u1.y, 0.0f));
           if constexpr (OUT != Out::Colour) {
             mw[q4 & 1] |= ((u0.x > 0.0f ? 1u : 0u) | (u0.y > 0.0f ? 2u : 0u) | (u1.x > 0.0f ? 4u : 0u) |
@@ -623,6 +799,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
             warp_arrive(&B.dfree[t & 1]);
           }
         }
+        if constexpr (ODD) {  // a NaN stays one, a number adds 0
+          if (q == 0) z0.x = 0.0f * v[0];
+        }
         const float4 a = l4[32 * (q / 8) + 2 * (q % 8)], b = l4[32 * (q / 8) + 2 * (q % 8) + 1];
         float2 u = add2(make_float2(v[2 * (HOLD ? q : q % 16)], v[2 * (HOLD ? q : q % 16) + 1]), make_float2(a.x, a.y));
         if constexpr (OUT != Out::Colour) {
@@ -664,9 +843,38 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
           base = __shfl_sync(0xffffffffu, base, 0);
           if (fix) w.rec_key[base + __popc(bal & ((1u << lane) - 1u))] = __float_as_uint(md.z);
         }
-        if (rid != 0xffffffffu)
-          w.rec_c[rid] = make_float4(sigmoid_f(z0.x + z0.y + o.x + b3s[0]), sigmoid_f(z1.x + z1.y + o.y + b3s[1]),
-                                     sigmoid_f(z2.x + z2.y + o.z + b3s[2]), md.y);
+        if (rid != 0xffffffffu) {
+          float4 c = make_float4(sigmoid_f(z0.x + z0.y + o.x + b3s[0]), sigmoid_f(z1.x + z1.y + o.y + b3s[1]),
+                                 sigmoid_f(z2.x + z2.y + o.z + b3s[2]), md.y);
+          if constexpr (ODD) {
+            if (isnan(c.x)) {
+              c.x = __uint_as_float(kOddColour);
+              B.marked = 1u;
+            }
+          }
+          w.rec_c[rid] = c;
+        }
+      }
+    }
+    if constexpr (ODD) {  // the marked samples again, a tile per warp at a time
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");  // every mark of E2's warps
+      const bool all = B.odd & kOddAll;
+      if (all || B.marked) {
+        for (uint32_t i = wid - kE2; i < n; i += kEpiWarps) {
+          const uint4 td = w.tile[t0 + i];
+          for (uint32_t k = 0; k < (td.y & 0xFFu); k += 32) {
+            uint32_t rid = 0xffffffffu;
+            if (k + lane < (td.y & 0xFFu)) rid = __float_as_uint(w.srt[td.x + k + lane].qd.x);
+            uint32_t todo = __ballot_sync(0xffffffffu, rid != 0xffffffffu && (all ||
+                                                       __float_as_uint(w.rec_c[rid].x) == kOddColour));
+            for (; todo; todo &= todo - 1u) {
+              const int s = __ffs(todo) - 1;
+              const float3 c = sample_f32(g, mlp, feat_, f16, w.srt + td.x + k + s,
+                                         !(B.odd & (kOddAll | kOddNan)));
+              if (lane == s) w.rec_c[rid] = make_float4(c.x, c.y, c.z, w.rec_c[rid].w);
+            }
+          }
+        }
       }
     }
   } else if (wid < kM) {
@@ -676,6 +884,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
     const uint32_t grp = (uint32_t)(wid - kG) / kGatWarps;  // takes tiles grp, grp + 2, ...
     const int C = CC ? CC : g.C, n_freq = NF ? NF : mlp.n_freq, Br = g.brick;
     float4* meta = (float4*)(sm + S::meta);
+    const bool tiny = ODD && (B.odd & kOddTiny);
+    (void)tiny;
     uint4 td = make_uint4(0u, 0u, 0u, 0u);
     float4 pw = make_float4(0.f, 0.f, 0.f, 0.f), qd = pw;
     auto fetch = [&](uint32_t i) {
@@ -714,6 +924,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
           gather<float, CC>(g, (const float*)feat_, i0, f, x);
       }
       if (i + 2 < n) fetch(i + 2);
+      if constexpr (ODD) {
+        if (tiny && any_huge<CC ? CC : kMaxC>(x)) x[0] = INFINITY;
+      }
       if (CC && NF && valid) encode<NF>(d, x + CC);
       if constexpr (OUT != Out::Colour) {  // ||x||^2 (the encoding's part below, if it is not in x yet)
 #pragma unroll
