@@ -175,7 +175,8 @@ cicero_status cicero_render_holes_batch(const cicero_grid *grid, const cicero_ml
 
 /* Workspace bytes for cicero_render / cicero_render_rays / cicero_render_holes with n_rays rays
  * (H*W, n_rays or max_holes).  Host query, allocates nothing.  For an FP16 grid that may be sampled
- * four times per vertex or more the size includes 16 bytes per vertex for a repacked density array; a
+ * four times per vertex or more the size includes 16 bytes per vertex for a repacked density array, made
+ * when the call's rays (as counted on the device) are many enough and run across the grid's x axis; a
  * workspace smaller by as much is accepted too, and the call then reads the density array as it is. */
 size_t cicero_render_workspace_size(const cicero_grid *grid, int n_rays, const cicero_sampling *sampling,
                                     const cicero_options *opt);

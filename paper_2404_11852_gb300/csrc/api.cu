@@ -211,12 +211,22 @@ cicero_status encode_brick_map(const cicero_grid* grid, const GridGeo& geo, cons
 
 static bool ws_ok(const void* ws) { return ws && (((uintptr_t)ws) & 255) == 0; }
 
-// Bytes of the packed voxels (k_pack) of an FP16 grid for a call that may composite up to Q samples: from
-// four such samples per vertex on.  Packing takes 2.6 ps per vertex (256^3 with a mask) and saves the march up
-// to 6.6 ps per composited sample, of which there are about 0.4 Q.
-static size_t pack_bytes(const cicero_grid* g, unsigned long long Q) {
+// Packed voxels (k_pack) of an FP16 grid: whether a call that may composite up to Q samples gets room for them
+// (from four per vertex on), and when it uses them.
+// What they save the march depends on the view: a warp's 32 samples lie along a ray, so their densities share
+// cache lines when the ray runs along x and do not when it runs across.  Over views around 64^3 .. 256^3 grids,
+// masked or not: 5 ps x (1 - |x component of the direction in voxels|) for every slot whose density is read.
+// Packing costs 12 us and, per vertex, 2.4 ps with a mask (15% of the cells) or 4.6 without.  So it pays from
+// pack_min such weighted slots on.  k_ray_setup adds them up on the device, where the number of rays (holes)
+// and their slots are known; k_pack and the march look.  With early stopping a ray counts for 64 slots at
+// most: on opaque scenes the march reads little more than the first 32 of hundreds (64 packs for fog from
+// half as many rays on as 32 would, and costs an opaque scene half of the packing at worst).
+static void plan_pack(const cicero_grid* g, const cicero_sampling* s, RenderPlan* p) {
   const unsigned long long verts = (unsigned long long)g->n[0] * g->n[1] * g->n[2];
-  return g->dtype == CICERO_F16 && Q >= 4 * verts && verts <= (1ull << 28) ? (size_t)verts * 16 : 0;
+  const bool room = g->dtype == CICERO_F16 && p->Q >= 4 * verts && verts <= (1ull << 28);
+  p->pack_bytes = room ? (size_t)verts * 16 : 0;
+  p->pack_cap = s->t_stop > 0.0f ? 64u : 65535u;
+  p->pack_min = room ? 2400000u + (uint32_t)((double)verts * (g->occ ? 0.48 : 0.92)) : 0u;
 }
 
 static cicero_status plan_render(const cicero_grid* grid, const cicero_mlp* mlp, int n_rays, const cicero_sampling* s,
@@ -243,7 +253,7 @@ static cicero_status plan_render(const cicero_grid* grid, const cicero_mlp* mlp,
   p->want_k = false;
   p->want_bwd = false;
   p->want_wg = false;
-  p->pack_bytes = pack_bytes(grid, Q);
+  plan_pack(grid, s, p);
   p->precision = opt ? opt->precision : CICERO_MLP_FP32;
   if (p->precision != CICERO_MLP_FP32 && p->precision != CICERO_MLP_BF16 && p->precision != CICERO_MLP_FP32_SPLIT)
     return fail(CICERO_ERR_INVALID_ARG, "precision");

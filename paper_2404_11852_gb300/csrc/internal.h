@@ -96,6 +96,8 @@ struct RenderWs {
   RayGeo* ray_geo;      // [R] geometry of each ray's samples
   struct RaySetup* setup;  // [R] per-ray setup of the march (ray, slots, active-slot mask, records)
   void* pack;           // [n2][n1][n0] voxels of eight FP16 corner densities (k_pack), or NULL
+  uint32_t pack_min;    // k_pack runs, and the march reads `pack`, when hdr[5] (k_ray_setup) is at least this
+  uint32_t pack_cap;    // slots of a ray that hdr[5] counts
   char* stage;          // per-sample operands of the MLP weight gradients (backward with d_mlp only; may be
                         // null): blocks of kStageBlock sorted samples, WgStage::bytes each (stage_col)
   int R, S, nb, max_tiles;
@@ -131,6 +133,7 @@ struct RenderPlan {
   bool want_k;
   bool want_bwd;
   size_t pack_bytes;  // of the packed voxels (RenderWs::pack); 0 = the march reads the density array itself
+  uint32_t pack_min, pack_cap;  // (RenderWs)
   bool want_wg;  // the backward stages the MLP weight gradients' operands (RenderWs::stage)
   cicero_precision precision;
   int mlp_groups;  // BF16 tensor-core MLP tiles in flight per SM (0 = as many as fit)

@@ -1,6 +1,7 @@
 // Memory-centric voxel-grid NeRF rendering (Sec. II-B stages, reordered as in Sec. IV-A).
 //
-//   Kp k_pack         (FP16 grids, many samples) the eight corner densities of every voxel side by side
+//   Kp k_pack         (FP16 grids, many samples across the x axis) the eight corner densities of every
+//                     voxel side by side
 //   K1 k_march        one warp per ray, 32 slots per step: Indexing, density gathering,
 //                     alpha, transmittance by a warp scan of sigma*delta, early stop; reserves an
 //                     upper bound of its records, emits one record (position, w, RIT key =
@@ -84,6 +85,8 @@ bool carve_render_ws(void* ws, size_t bytes, const RenderPlan& plan, RenderWs* w
   w->srt = (SrtRec*)take(32 * Q);
   w->setup = (RaySetup*)take(kRaySetupBytes * R);
   w->pack = p.pack_bytes ? take(p.pack_bytes) : nullptr;
+  w->pack_min = p.pack_min;
+  w->pack_cap = p.pack_cap;
   w->R = p.R;
   w->S = p.S;
   w->nb = p.nb;
@@ -353,12 +356,17 @@ struct __align__(16) Packed {
 // are left unwritten, no sample that the index test accepts reads them), so that the march reads a
 // sample's eight corners with one 16-byte load.  The march is bound by L1 wavefronts, one for every line
 // that a warp's 32 scattered samples touch, and eight scattered 2-byte loads per sample were 76% of its
-// time: 62.5 M samples of a 256^3 grid 1208 -> 797 us of march, for 43 us of packing.  (FP32 voxels of 32
+// time: 62.5 M samples of a 256^3 grid 1208 -> 797 us of march, for 43 us of packing, in a view across x.  (FP32 voxels of 32
 // bytes save what packing them costs: 214 -> 198 us of march for 12 of packing on 18.4 M samples of a
 // 96 x 113 x 80 grid.)  Thread (x, y) walks up kPackZ voxels and keeps the upper plane's values for the next.
+// Nothing is packed when the call's rays do not make up for it (plan_pack in api.cu): a hole call of 640 rays
+// on an unmasked 256^3 grid took 26 us of march, 104 with the packing, 31 with the kernel that only looks.
 constexpr int kPackZ = 16;
-__global__ void __launch_bounds__(256) k_pack(GridGeo g, const __half* __restrict__ dens, Packed* pack) {
+__device__ __forceinline__ bool use_pack(const RenderWs& w) { return w.hdr[5] >= w.pack_min; }
+__global__ void __launch_bounds__(256) k_pack(GridGeo g, const __half* __restrict__ dens, RenderWs w) {
   dependents_sync();
+  if (!use_pack(w)) return;
+  Packed* pack = (Packed*)w.pack;
   const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 8 + (threadIdx.x >> 5);
   if (x >= g.n[0] - 1 || y >= g.n[1] - 1) return;
   const size_t nx = g.n[0], nxy = nx * g.n[1];
@@ -622,6 +630,8 @@ __global__ void __launch_bounds__(256) k_ray_setup(GridGeo g, Samp s, RaySrc src
                                                    const int* __restrict__ bases, int n_jobs, int R_batch, RenderWs w) {
   dependents_sync();
   __shared__ RaySetup sq[256];
+  const bool weigh = !BATCH && w.pack;  // add up what packed voxels would save (plan_pack in api.cu)
+  float saved = 0.0f;
   const int R = BATCH ? R_batch : ray_count(src);
   for (long long r0 = (long long)blockIdx.x * 256; r0 < R; r0 += (long long)gridDim.x * 256) {
     const long long r = r0 + threadIdx.x;
@@ -652,6 +662,10 @@ __global__ void __launch_bounds__(256) k_ray_setup(GridGeo g, Samp s, RaySrc src
       rg.ot = make_float4(q.o[0], q.o[1], q.o[2], q.t0);
       rg.dd = make_float4(q.d[0], q.d[1], q.d[2], q.dt);
       w.ray_geo[r] = rg;
+      if (weigh) {
+        const float vx = q.d[0] * g.inv_h[0], vy = q.d[1] * g.inv_h[1], vz = q.d[2] * g.inv_h[2];
+        saved += (float)min((uint32_t)q.nact, w.pack_cap) * (1.0f - fabsf(vx) * rsqrtf(vx * vx + vy * vy + vz * vz));
+      }
     }
     __syncthreads();
     const int n = (int)min((long long)256, (long long)R - r0);
@@ -659,6 +673,15 @@ __global__ void __launch_bounds__(256) k_ray_setup(GridGeo g, Samp s, RaySrc src
     uint32_t* to = reinterpret_cast<uint32_t*>(w.setup + r0);
     for (int i = threadIdx.x; i < n * kSetupWords; i += 256) to[i] = from[i];
     __syncthreads();
+  }
+  if (weigh) {  // whole slots per thread: the sum does not depend on its order
+    uint32_t* block_sum = reinterpret_cast<uint32_t*>(sq);
+    if (threadIdx.x == 0) *block_sum = 0u;
+    __syncthreads();
+    const uint32_t warp_sum_ = __reduce_add_sync(0xffffffffu, (uint32_t)fmaxf(saved, 0.0f));
+    if ((threadIdx.x & 31) == 0) atomicAdd(block_sum, warp_sum_);
+    __syncthreads();
+    if (threadIdx.x == 0 && *block_sum) atomicAdd(&w.hdr[5], *block_sum);
   }
 }
 
@@ -668,17 +691,15 @@ __device__ __forceinline__ uint32_t setup_word(const RenderWs& w, long long r, i
 }
 
 // K1: one warp per ray, rays r = warp + i nwarps; each ray's setup (from K0) is staged in shared
-// memory, the next ray's loaded while the current one marches.
+// memory, the next ray's loaded while the current one marches.  setup, slot_list: of the block's 8 warps.
 template <typename T, bool EXTRA, bool PACKED>
-__global__ void __launch_bounds__(256, 4) k_march(GridGeo g, Samp s, RaySrc src, const T* __restrict__ dens,
-                                               RenderWs w, OutBufs out) {
-  dependents_sync();
+__device__ __forceinline__ void march_rays(const GridGeo& g, const Samp& s, const RaySrc& src, const T* __restrict__ dens,
+                                           const RenderWs& w, const OutBufs& out, RaySetup* setup,
+                                           uint8_t (*slot_list)[kMaskSlots]) {
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
   const int R = ray_count(src);
-  __shared__ RaySetup setup[8];
-  __shared__ uint8_t slot_list[8][kMaskSlots];
   const int wb = threadIdx.x >> 5;
   uint32_t next = warp < R ? setup_word(w, warp, lane) : 0u;
   for (long long r = warp; r < R; r += nwarps) {
@@ -692,6 +713,17 @@ __global__ void __launch_bounds__(256, 4) k_march(GridGeo g, Samp s, RaySrc src,
                              slot_list[wb]);
     __syncwarp();  // the setup slot is free for the next ray
   }
+}
+
+// MAY_PACK: the workspace has room for packed voxels; whether k_pack filled it is the call's to decide.
+template <typename T, bool EXTRA, bool MAY_PACK>
+__global__ void __launch_bounds__(256, 4) k_march(GridGeo g, Samp s, RaySrc src, const T* __restrict__ dens,
+                                               RenderWs w, OutBufs out) {
+  dependents_sync();
+  __shared__ RaySetup setup[8];
+  __shared__ uint8_t slot_list[8][kMaskSlots];
+  if (MAY_PACK && use_pack(w)) march_rays<T, EXTRA, MAY_PACK>(g, s, src, dens, w, out, setup, slot_list);
+  else march_rays<T, EXTRA, false>(g, s, src, dens, w, out, setup, slot_list);
 }
 
 // K2: exclusive scan of the brick histogram and the list of tiles (<= kTile samples of one brick).
@@ -1542,7 +1574,7 @@ cicero_status run_render(const cicero_grid* grid, const MlpPtrs& mlp, const Rend
     const float* d32 = (const float*)grid->density;
     if (ws.pack) {
       const dim3 gp((geo.n[0] + 30) / 32, (geo.n[1] + 6) / 8, (geo.n[2] - 2) / kPackZ + 1);
-      launch_kernel(k_pack, gp, 256, 0, st, geo, d16, (Packed*)ws.pack);
+      launch_kernel(k_pack, gp, 256, 0, st, geo, d16, ws);
       count_launches(1);
       extra ? march(k_march<__half, true, true>, d16) : march(k_march<__half, false, true>, d16);
     } else if (f16) {
