@@ -529,6 +529,14 @@ struct cicero_batch {
 
 namespace cicero {
 
+size_t render_ws_size(const cicero_grid* grid, int n_rays, const cicero_sampling* s, const cicero_options* opt,
+                      bool pack) {
+  RenderPlan plan;
+  if (plan_render(grid, nullptr, n_rays, s, opt, &plan, false) != CICERO_OK) return 0;
+  if (!pack) plan.pack_bytes = 0;
+  return render_ws_bytes(plan);
+}
+
 static size_t batch_ws_bytes(const BatchPlan& b) { return batch_table_bytes(b.n_jobs) + render_ws_bytes(b.plan); }
 
 }  // namespace cicero
@@ -616,9 +624,7 @@ cicero_status cicero_render_holes_batch(const cicero_grid* grid, const cicero_ml
 
 size_t cicero_render_workspace_size(const cicero_grid* grid, int n_rays, const cicero_sampling* sampling,
                                     const cicero_options* opt) {
-  RenderPlan plan;
-  if (plan_render(grid, nullptr, n_rays, sampling, opt, &plan, false) != CICERO_OK) return 0;
-  return render_ws_bytes(plan);
+  return render_ws_size(grid, n_rays, sampling, opt, true);
 }
 
 size_t cicero_build_rit_workspace_size(const cicero_grid* grid, const cicero_camera* cam,
@@ -672,7 +678,7 @@ cicero_status cicero_autotune_brick(const cicero_grid* grid, const cicero_mlp* m
   for (int i = 0; i < 3; i++) {
     if (ms) ms[i] = -1.0f;
     cicero_options opt = {precision, cand[i], 0};
-    const size_t need = cicero_render_workspace_size(grid, cam ? cam->width * cam->height : 0, sampling, &opt);
+    const size_t need = render_ws_size(grid, cam ? cam->width * cam->height : 0, sampling, &opt, false);
     if (need == 0 || need > ws_bytes) continue;
     // one untimed render (first use of the kernel), then one timed render
     if (cicero_render(grid, mlp, cam, sampling, &opt, rgb, depth, nullptr, nullptr, workspace, ws_bytes, stream) !=

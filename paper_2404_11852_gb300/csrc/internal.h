@@ -149,6 +149,8 @@ struct OutBufs {
 };
 
 size_t render_ws_bytes(const RenderPlan& p);
+// cicero_render_workspace_size, with or without the room for packed voxels, which a render can do without
+size_t render_ws_size(const cicero_grid* grid, int n_rays, const cicero_sampling* s, const cicero_options* opt, bool pack);
 bool carve_render_ws(void* ws, size_t bytes, const RenderPlan& p, RenderWs* out);
 
 // grid/sampling validation and geometry (api.cu)

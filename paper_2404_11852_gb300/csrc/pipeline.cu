@@ -68,20 +68,22 @@ struct PipeLayout {
 
 static size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// pack: with room for packed voxels in the renders' workspaces, which they can do without
 static cicero_status pipe_layout(const cicero_grid* grid, const cicero_camera* cam, const cicero_sampling* samp,
-                                 const cicero_options* opt, int window, long long hole_records, PipeLayout* L) {
+                                 const cicero_options* opt, int window, long long hole_records, bool pack,
+                                 PipeLayout* L) {
   if (!grid || !cam || !samp || !opt) return fail(CICERO_ERR_INVALID_ARG, "a pipeline argument is NULL");
   if (window < 1 || window > kMaxWarpViews) return fail(CICERO_ERR_INVALID_ARG, "window must be 1..32");
   if (hole_records < 0) return fail(CICERO_ERR_INVALID_ARG, "hole_records must be >= 0");
   const size_t R = (size_t)cam->width * cam->height;
-  L->ws_ref_bytes = cicero_render_workspace_size(grid, (int)R, samp, opt);
+  L->ws_ref_bytes = render_ws_size(grid, (int)R, samp, opt, pack);
   cicero_camera tc[kMaxWarpViews];
   for (int v = 0; v < window; v++) tc[v] = *cam;
   L->ws_warp_bytes = cicero_warp_batch_workspace_size(tc, window);
   cicero_options oh = *opt;
   oh.max_records = hole_records;
   if ((long long)R * window > 0x7fffffffll) return fail(CICERO_ERR_UNSUPPORTED, "window x pixels must fit 31 bits");
-  L->ws_holes_bytes = cicero_render_workspace_size(grid, (int)(R * window), samp, &oh);
+  L->ws_holes_bytes = render_ws_size(grid, (int)(R * window), samp, &oh, pack);
   if (!L->ws_ref_bytes || !L->ws_warp_bytes || !L->ws_holes_bytes) return fail(CICERO_ERR_INVALID_ARG, cicero_last_error());
   size_t o = 0;
   auto take = [&](size_t n) {
@@ -180,7 +182,7 @@ size_t cicero_pipeline_workspace_size(const cicero_grid* grid, const cicero_came
                                       const cicero_sampling* sampling, const cicero_options* opt, int window,
                                       long long hole_records) {
   PipeLayout L;
-  return pipe_layout(grid, cam, sampling, opt, window, hole_records, &L) == CICERO_OK ? L.total : 0;
+  return pipe_layout(grid, cam, sampling, opt, window, hole_records, true, &L) == CICERO_OK ? L.total : 0;
 }
 
 cicero_status cicero_pipeline_create(const cicero_grid* grid, const cicero_mlp* mlp, const cicero_camera* cam,
@@ -190,7 +192,8 @@ cicero_status cicero_pipeline_create(const cicero_grid* grid, const cicero_mlp* 
   if (!out || !mlp) return fail(CICERO_ERR_INVALID_ARG, "out/mlp is NULL");
   *out = nullptr;
   PipeLayout L;
-  cicero_status st = pipe_layout(grid, cam, sampling, opt, window, hole_records, &L);
+  cicero_status st = pipe_layout(grid, cam, sampling, opt, window, hole_records, true, &L);
+  if (st == CICERO_OK && L.total > ws_bytes) st = pipe_layout(grid, cam, sampling, opt, window, hole_records, false, &L);
   if (st != CICERO_OK) return st;
   if (!workspace || ((uintptr_t)workspace & 255)) return fail(CICERO_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
   if (L.total > ws_bytes) return fail(CICERO_ERR_WORKSPACE_TOO_SMALL, "workspace too small for the pipeline");

@@ -55,3 +55,33 @@ def test_packing_follows_the_rays(cc, az, holes, occ, t_stop, packed):
             assert bool((tail != 0xA5).any()) == packed
         got.append((rgb, depth))
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
+def test_workspaces_without_the_voxels(cc):
+    """The autotuner and the pipeline take a workspace without room for the packed voxels, as a render does, and
+    give the same images; one smaller still is refused."""
+    import torch
+    n, w, S, window = 48, 160, 64, 3
+    g = cc.DeviceGrid.from_host(scenes.make_grid(n, 4, 6, seed=7, dtype="float16"))
+    m = cc.DeviceMlp.from_host(scenes.make_mlp(4, seed=8))
+    cams = [scenes.orbit_camera(w, w, az_deg=60.0 + k) for k in range(5)]
+    cds = [cc.camera_from(c) for c in cams]
+    sd, R, voxels = cc.sampling(0.5, 2.5, S, 0.0, 1e-3), w * w, (16 * n ** 3 + 255) // 256 * 256
+    need = max(cc.cicero_render_workspace_size(g.desc, R, sd, cc.options(cc.MLP_BF16, b)) for b in (4, 8, 16))
+    rgb, depth = torch.empty(R, 3, device="cuda"), torch.empty(R, device="cuda")
+    best, ms = cc.cicero_autotune_brick(g.desc, m.desc, cds[0], sd, cc.MLP_BF16, rgb, depth, cc.workspace(need - voxels))
+    assert best in (4, 8, 16) and all(t > 0 for t in ms.values())
+    opt, records = cc.options(cc.MLP_BF16, 4), window * R * S
+    need = cc.cicero_pipeline_workspace_size(g.desc, cds[0], sd, opt, window, records)
+    out = []
+    for bytes_ in (need, need - 3 * voxels):
+        frames = [torch.empty(R, 3, device="cuda") for _ in cds], [torch.empty(R, device="cuda") for _ in cds]
+        ws = cc.workspace(bytes_)
+        pipe = cc.Pipeline(g.desc, m.desc, cds[0], sd, opt, window, records, 180.0, ws)
+        pipe.run(cds, *frames)
+        torch.cuda.synchronize()
+        out.append(frames)
+    for a, b in zip(out[0][0] + out[0][1], out[1][0] + out[1][1]):
+        assert torch.equal(a, b)
+    with pytest.raises(cc.CiceroError):
+        cc.Pipeline(g.desc, m.desc, cds[0], sd, opt, window, records, 180.0, cc.workspace(need - 3 * voxels - 256))
