@@ -76,14 +76,15 @@ __device__ __forceinline__ bool gsync_and(int g, bool v) {
   return r != 0;
 }
 
-// 8 consecutive weights
+// 8 consecutive weights.  Ordinary loads: k_mlp_eval_bf16 is the first kernel of its call, and the caller's
+// last one may still have been writing the weights while it started (dependents_sync).
 __device__ __forceinline__ void load8(const float* p, bool vec, float* v) {
   if (vec) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
     v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
   } else {
 #pragma unroll
-    for (int j = 0; j < 8; j++) v[j] = __ldg(p + j);
+    for (int j = 0; j < 8; j++) v[j] = p[j];
   }
 }
 
