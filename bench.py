@@ -8,7 +8,7 @@ its holes (Eq. 4).  value = 16 target frames x steps x ranks / time.  The plain 
 of the same frame is measured beside it.  With --gpus N every rank renders its own window
 (different orbit azimuth): weak scaling, no collective on the data path.
 
-Prints one JSON line (rank 0).  --impl reference times the FP64 CPU oracle on a bounded sample of
+Prints one JSON line (rank 0); --detail FILE writes the full record.  --impl reference times the FP64 CPU oracle on a bounded sample of
 the same workload instead.
 """
 from __future__ import annotations
@@ -58,6 +58,7 @@ def parse():
                    help="small: one 320x320 reference frame (BF16 and FP32) and two targets, for profilers; "
                         "backward: the differentiation workload alone")
     p.add_argument("--brick", type=int, default=4, help="brick size of the small case")
+    p.add_argument("--detail", metavar="FILE", help="also write the full record (every workload's figures) as JSON")
     return p.parse_args()
 
 
@@ -891,6 +892,49 @@ def sparw_small_scene(cc, torch, dev, n_pix=1024, opaque=False):
 
 
 # ---------------------------------------------------------------------------------------------
+# the printed line
+
+# what the line takes over from the record as it is, and single figures of the other workloads
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "plain_fp32_fps", "bf16_full_fps", "fp32_split_full_fps",
+             "msamples_per_s_bf16_full", "msamples_per_s_fp32_full", "active_samples_per_frame",
+             "fraction_rays_marched_targets", "brick", "roofline", "quality", "e2e", "gpu_launches", "clocks")
+LINE_FIGURES = {"backward_ms": ("config_backward", "backward_ms"),
+                "backward_with_mlp_weights_ms": ("config_backward", "backward_with_mlp_weights_ms"),
+                "small_scene_target_fps": ("config_sparw_small_scene", "target_fps"),
+                "opaque_scene_target_fps": ("config_sparw_opaque_scene", "target_fps"),
+                "batch_48_jobs_ms": ("config_batched", "batch_ms"),
+                "batch_one_call_per_job_ms": ("config_batched", "one_call_per_job_ms"),
+                "hash_grid_fps": ("config_hash_grid", "fps")}
+LINE_BYTES = 4096
+
+
+def _short(x):
+    if isinstance(x, dict):
+        return {k: _short(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [_short(v) for v in x]
+    return float(f"{x:.7g}") if isinstance(x, float) else x
+
+
+def headline(record: dict) -> str:
+    """The benchmark's one line: a few kilobytes, whatever the record holds (its readers may keep only the
+    last ones of the output); --detail writes the whole record."""
+    line = {k: record[k] for k in LINE_KEYS if k in record}
+    if "stages" in record:
+        line["stage_ms"] = {k: v["ms_per_step"] for k, v in record["stages"].items()}
+    if record.get("cpu_baseline"):
+        line["cpu_baseline"] = {k: v for k, v in record["cpu_baseline"].items() if k != "threads"}
+    line["workloads"] = {k: record[w][f] for k, (w, f) in LINE_FIGURES.items() if f in record.get(w, {})}
+    s = json.dumps(_short(line))
+    for k in ("workloads", "stage_ms", "quality", "roofline"):  # what the line can do without
+        if len(s) > LINE_BYTES:
+            line.pop(k, None)
+            s = json.dumps(_short(line))
+    return s
+
+
+# ---------------------------------------------------------------------------------------------
 # GPU leg
 
 
@@ -1178,7 +1222,10 @@ def main():
             "clocks": clk.summary(),
             **others,
         }
-        print(json.dumps(line), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as f:
+                json.dump(line, f, indent=1)
+        print(headline(line), flush=True)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()
