@@ -768,12 +768,14 @@ __device__ __forceinline__ void block_exscan2(uint32_t a, uint32_t b, uint32_t* 
 
 // Where a key's scatter cursor stands.  The cursors of neighbouring bricks share 128-byte lines, and a
 // line's atomics all go to one L2 slice: on a small scene whose samples lie in a few hundred bricks one
-// slice took 8 times the average (60% busy, the others 4%).  From 1025 to 16384 bricks the cursors are
-// spread: octant by octant, neighbouring bricks cursor_step entries apart (bucketing of a 64^3 scene with bricks of 4,
-// 400x304: 199 -> 163 us a frame; of 2,100 bricks 266 -> 260).  Larger tables spread by themselves and gain
-// more from a ray's consecutive keys lying together (256^3, bricks of 4: 643 -> 702 us spread).
+// slice took 8 times the average (60% busy, the others 4%).  From 1025 to 12288 bricks the cursors are
+// spread: octant by octant, neighbouring bricks cursor_step entries apart.  Larger tables spread by themselves and
+// gain more from a ray's consecutive keys lying together.  Bucketing of two fog scenes, 800x800 x 128 slots,
+// bricks of 4, together and spread, in us: 1,331 bricks 1104 -> 788 and 1067 -> 628; 4,913 846 -> 831 and 917 ->
+// 644; 9,261 919 -> 908 and 772 -> 715; 12,167 888 -> 928 and 768 -> 717; 15,625 944 -> 1018 and 758 -> 755; 262,144
+// (256^3 frame) 643 -> 702.
 __device__ __forceinline__ uint32_t cursor_step(uint32_t nb) {  // coprime to nb (a prime that does not divide it)
-  return nb <= 1024u || nb > 16384u ? 0u : (nb % 1009u ? 1009u : 1013u);
+  return nb <= 1024u || nb > 12288u ? 0u : (nb % 1009u ? 1009u : 1013u);
 }
 __device__ __forceinline__ uint32_t cursor_at(uint32_t key, uint32_t nb, uint32_t step) {
   return step ? (key % kOctants) * nb + ((key / kOctants) * step) % nb : key;
