@@ -221,15 +221,18 @@ __device__ __forceinline__ uint32_t h1_col(int k, uint32_t i) { return k == 0 ? 
 // with the CTA's tiles.  E1 lets a NaN of its first unit through the ReLU (all units are NaNs then: an input
 // that cannot be split), layer 2's sums carry it (or that of an h1 that cannot be split), and E2 carries it
 // into the colour.  A NaN among the weights or biases of a unit marks nothing: the unit is 0 in both chains and
-// is taken out of the operands (drop_nan_units).
+// is taken out of the operands (drop_nan_units).  One in layer 3's first row makes every first colour a NaN, as
+// it should be, and no mark can be told from it (kOddBlind).
 // A weight or a bias of layer 1 from kHuge on marks every sample.  One below kTiny has parts below BF16's smallest number and is off
 // by up to 2^-134, too little to count beside operands below kHuge; with such weights G and E1 mark the
 // samples of larger ones.
-// A render without any of these pays an instruction or two per thread and tile, and the look at the weights
-// (62.5 M samples 8.78 -> 8.85 ms, a 64x64 frame the same); a sample taken again costs an SM ~5,000 clocks.
+// A render without any of these pays a few instructions per thread and tile, the look at the weights and what the
+// code below does to the roles' registers: 0.98 to 1.03 of the time without, over five FP32 calls from 85 us to 2.8
+// ms (a mean of 1.00; 62.5 M samples 8.78 -> 8.85 ms).  (Flags from an earlier kernel and the samples taken again by
+// one of its own: the same within 1%.)  A sample taken again costs an SM ~5,000 clocks.
 constexpr float kHuge = 0x1p100f, kTiny = 0x1p-109f;
 constexpr uint32_t kOddColour = 0x7FC0BABEu;  // a NaN that no arithmetic returns
-enum Odd : uint32_t { kOddNan = 1, kOddAll = 2, kOddTiny = 4 };
+enum Odd : uint32_t { kOddNan = 1, kOddAll = 2, kOddTiny = 4, kOddBlind = 8 };
 __device__ __forceinline__ float relu_nan(float v) {
   float r;
   asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(v));
@@ -266,8 +269,10 @@ __device__ __forceinline__ uint32_t odd_parameters(const char* sm) {
                (lo < (__float_as_uint(kTiny) >> 16) - 1u ? kOddTiny : 0u);
   for (int i = threadIdx.x; i < 5 * kHidden; i += kThreads) {
     const float v = ((const float*)(sm + S::b1))[i];
-    f |= (isnan(v) ? kOddNan : 0u) | (i < kHidden && fabsf(v) >= kHuge ? kOddAll : 0u);
+    f |= (isnan(v) ? (i >= kHidden && (i & 6) == 2 ? kOddBlind : kOddNan) : 0u) |
+         (i < kHidden && fabsf(v) >= kHuge ? kOddAll : 0u);
   }
+  if (isnan(((const float*)(sm + S::b3))[0])) f |= kOddBlind;
   return f;
 }
 
@@ -859,7 +864,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(GridGeo g, MlpPtrs ml
     if constexpr (ODD) {  // the marked samples again, a tile per warp at a time
       asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");  // every mark of E2's warps
       const bool all = B.odd & kOddAll;
-      if (all || B.marked) {
+      if (all || (B.marked && !(B.odd & kOddBlind))) {
         for (uint32_t i = wid - kE2; i < n; i += kEpiWarps) {
           const uint4 td = w.tile[t0 + i];
           for (uint32_t k = 0; k < (td.y & 0xFFu); k += 32) {

@@ -86,3 +86,23 @@ def test_fp32_operands_without_bf16_parts(cc, orc, kind, C):
         assert (~keep).sum() <= 3
         out, ref = ({k: v[keep] for k, v in o.items()} for o in (out, ref))
     check_render(out, ref, TOL)
+
+
+@pytest.mark.parametrize("kind", ["big_feature", "inf_feature"])
+def test_wide_backward_recompute(cc, orc, kind):
+    """The backward of more than 16 channels takes its colours from the same kernel: the density's gradient."""
+    import torch
+    C, R = 20, 200
+    g, m = scene(kind, C)
+    o, d = scenes.random_rays(R, seed=77)
+    sp = scenes.Sampling(near=0.5, far=2.5, n_samples=24, t_stop=0.0)
+    grad = np.random.default_rng(5).standard_normal((R, 3)).astype(np.float32)
+    want = orc.backward(g, m, sp, grad, rays=(o, d))[0].ravel()
+    assert np.isfinite(want).all()
+    gd, md, sd = cc.DeviceGrid.from_host(g), cc.DeviceMlp.from_host(m), cc.sampling_from(sp)
+    dd, df = torch.zeros(g.density.shape, device="cuda"), torch.zeros(g.features.shape, device="cuda")
+    ws = cc.workspace(cc.cicero_backward_workspace_size(gd.desc, R, sd))
+    cc.cicero_render_backward(gd.desc, md.desc, torch.from_numpy(o).cuda(), torch.from_numpy(d).cuda(), sd,
+                              torch.from_numpy(grad).cuda(), dd, df, None, ws)
+    cc.cicero_workspace_status(ws)
+    assert np.abs(dd.cpu().double().numpy().ravel() - want).max() <= 1e-3 * np.abs(want).max()  # the path's tolerance
