@@ -36,11 +36,11 @@ HOLE_RECORDS = 128_000_000  # record capacity of the batched hole render (6.7 GB
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one k_gather_mlp_bf16 launch on the
 # 800x800 reference frame, from a one-pass ncu capture of this benchmark, and the SHA-1 of the
 # kernel sources it was taken on; the roofline reports it only while those sources are unchanged.
-GATHER_TRAFFIC = {"bytes": 2742457856 + 1359033856, "sources_sha1": "9d9cadcd8128ab014fadc07c6f8d80e7c5cd154e"}
+GATHER_TRAFFIC = {"bytes": 2743529216 + 1359711744, "sources_sha1": "e7a3b82d3547b5c3abae607ca51a8b083dfd2629"}
 GATHER_SOURCES = ("mlp_tc.cu", "common.cuh", "internal.h")
 # shared-memory wavefronts per composited sample of the BF16 gather (LSU loads + LSU stores +
 # tensor-core operand reads, ncu on the 320x320 case), valid for the sources hashed above
-GATHER_SMEM_WAVEFRONTS_PER_SAMPLE = (24302060 + 31859312 + 67379200) / 10312421
+GATHER_SMEM_WAVEFRONTS_PER_SAMPLE = (25130108 + 32123273 + 67379200) / 10312421
 
 
 def parse():
@@ -135,16 +135,16 @@ def stage_roofline(stages, pk, R, n_holes, ref_samples, hole_samples):
     """Per stage of one SpaRW window: algorithmic bytes (or FLOP), achieved rate over the stage's
     device time, and the fraction of the measured peak of the resource that bounds it.
 
-    Bytes counted: march, per composited sample its record (brick id 4 B + position/weight 16 B)
-    and per ray its header and depth (36 B); bucket, per record 20 B read + 32 B written (the Ray
+    Bytes counted: march, per composited sample its record (key 4 B, weight 4 B, slot 2 B)
+    and per ray its header and depth (36 B); bucket, per record 10 B read + 32 B written (the Ray
     Index Table payload) + 24 B of ray header per ray; gather + MLP, 43,520 FLOP per sample;
     composite, per sample 16 B read + per ray 28 B; warp splat, per reference pixel 16 B read +
     8 B of depth-key atomic per target; warp resolve, ~29 B per target pixel."""
     rays = R + n_holes
     samples = ref_samples + hole_samples
     work = {
-        "march": ("issue", 20.0 * samples + 36.0 * rays),
-        "bucket": ("hbm", 52.0 * samples + 24.0 * rays),
+        "march": ("issue", 10.0 * samples + 36.0 * rays),
+        "bucket": ("hbm", 42.0 * samples + 24.0 * rays),
         "gather_mlp": ("tensor", float(FLOP_PER_SAMPLE) * samples),
         "composite": ("hbm", 16.0 * samples + 28.0 * rays),
         "warp_splat": ("hbm", (16.0 + 8.0 * N_TARGETS) * R),
