@@ -329,8 +329,8 @@ __device__ __forceinline__ void encode_dir(const float d[3], int n_freq, float* 
   }
 }
 
-// Programmatic dependent launch: every kernel of a call but the composite is launched while its
-// predecessor on the stream may still run (launch_kernel in internal.h).  A kernel calls
+// Programmatic dependent launch: every kernel of a call but the composite and the void test of several
+// views is launched while its predecessor on the stream may still run (launch_kernel in internal.h).  A kernel calls
 // dependents_sync() before it touches anything a predecessor wrote or still reads: it waits until the
 // predecessor is complete and its writes visible, and only then lets its own successor start.  So
 // whatever runs before the call (weights into shared memory, barriers, tensor memory) may read what the
