@@ -36,7 +36,7 @@ HOLE_RECORDS = 128_000_000  # record capacity of the batched hole render (6.7 GB
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one k_gather_mlp_bf16 launch on the
 # 800x800 reference frame, from a one-pass ncu capture of this benchmark, and the SHA-1 of the
 # kernel sources it was taken on; the roofline reports it only while those sources are unchanged.
-GATHER_TRAFFIC = {"bytes": 2743529216 + 1359711744, "sources_sha1": "e7a3b82d3547b5c3abae607ca51a8b083dfd2629"}
+GATHER_TRAFFIC = {"bytes": 2744288256 + 1360022784, "sources_sha1": "405872281344e22e9ce2e1249bd7c7c07175538c"}
 GATHER_SOURCES = ("mlp_tc.cu", "common.cuh", "internal.h")
 # shared-memory wavefronts per composited sample of the BF16 gather (LSU loads + LSU stores +
 # tensor-core operand reads, ncu on the 320x320 case), valid for the sources hashed above
