@@ -182,7 +182,8 @@ size_t cicero_render_workspace_size(const cicero_grid *grid, int n_rays, const c
                                     const cicero_options *opt);
 
 /* Brick-size autotuner: renders `cam` once untimed and once timed with bricks of 4, 8 and 16
- * voxels (each size that fits `ws_bytes` and the kernels' shared memory) and returns the fastest in
+ * voxels (each size that fits `ws_bytes`, with or without room for the repacked density array, and
+ * the kernels' shared memory) and returns the fastest in
  * *best_brick; ms[3] (may be NULL) receives the timed milliseconds (-1 = not tried).  rgb and depth
  * (device, [H*W][3] and [H*W]) are scratch.  Size the workspace with brick 4, the largest.
  * Synchronises `stream` (it times with CUDA events), unlike every other call. */
@@ -323,7 +324,9 @@ cicero_status cicero_reference_poses(const cicero_camera *targets, int n_frames,
  *
  * The workspace holds two reference frames and their render workspaces (opt applies to them),
  * scratch for one window's hole masks and lists, and the hole-batch workspace of `hole_records`
- * records (opt's max_records for the hole batch).  The handle is host memory owned by the
+ * records (opt's max_records for the hole batch).  A workspace without the room that these render
+ * workspaces have for a repacked density array (cicero_render_workspace_size) is taken too; the
+ * renders then read the density array as it is.  The handle is host memory owned by the
  * caller; one run at a time per pipeline (the previous run's work is waited for on the streams,
  * not on the host).  targets [n_frames] is a host array; rgb / depth are host arrays of n_frames
  * device pointers ([H*W][3] / [H*W]; depth may be NULL).
